@@ -59,13 +59,17 @@ typedef enum { SCD_FP32 = 0, SCD_SPLIT_BF16 = 1 } scd_precision;
  * PERSISTENT: one persistent launch that runs the channeliser + CDP and then the column and
  *   row passes channel group by channel group through small rotating slots (so each group's
  *   intermediate is read back from L2).
- * FUSED: two kernels: the channeliser, the channel-data product and the strip transform's
- *   first pass in one (the product X_g never leaves the chip), the second pass in the other.
- *   Where its tiles do not fit the sizes (FP32 form; Np in {64, 128, 256}, N = M1 M2 with
- *   M1 = 64, 128 or 256, Np <= M2 <= 2048: N = 2^12..2^19 at Np = 64, 2^13..2^19 at
- *   Np = 128, 2^14..2^18 at Np = 256), the call runs the STAGES kernels instead.
+ * FUSED: the product X_g never reaches memory.  An auto estimate runs in the lag domain: the
+ *   strip transforms of the lag products x[n + m] conj(x[n]), m >= 0, then one Np-point
+ *   transform over the lags per frequency (half the strip transforms, by conjugate symmetry).  A
+ *   cross or conjugate estimate runs two kernels: the channeliser, the channel-data product
+ *   and the strip transform's first pass in one, the second pass in the other.
+ *   Where the latter's tiles do not fit the sizes (FP32 form; Np in {64, 128, 256}, N = M1 M2
+ *   with M1 = 64, 128 or 256, Np <= M2 <= 2048: N = 2^12..2^19 at Np = 64, 2^13..2^19 at
+ *   Np = 128, 2^14..2^18 at Np = 256), a call that asks for FUSED runs the STAGES kernels.
  * AUTO: the choice scd_ssca_tune measured fastest for (N, Np, precision) on this GPU model
- *   (in this process, or from the SCD_TUNE_CACHE file); if never tuned, FUSED where it fits,
+ *   (in this process, or from the SCD_TUNE_CACHE file); if never tuned, in the FP32 form the
+ *   lag-domain kernels for an auto estimate of any power-of-two N, else FUSED where it fits,
  *   else STAGES. */
 typedef enum {
   SCD_SCHEDULE_AUTO = 0,
@@ -89,7 +93,9 @@ typedef struct {
    * FFT; 3 for a cross or conjugate estimate: channeliser of x, of y, pair FFT); scd_ssca 3
    * with the STAGES schedule (channeliser + CDP, column pass, row pass), 2 with FUSED
    * (channeliser + CDP + first pass, second pass) or 1 with PERSISTENT (AUTO resolves to
-   * one of these); each map and profile 1. */
+   * one of these); each map and profile 1.  The lag-domain kernels record as many events as the
+   * call did before there were any: 3 at FUSED's sizes (before, between the strip and the channel
+   * transforms, after), 4 at the others (also between the strip's two passes). */
   void** stage_events;
   int32_t n_stage_events;
   int32_t schedule;         /* scd_ssca only: scd_schedule */

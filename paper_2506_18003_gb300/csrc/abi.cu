@@ -152,11 +152,13 @@ scd_status scd_fam(const void* x, int64_t N, int32_t Np, int32_t L, int32_t P, c
   return SCD_OK;
 }
 
-scd_status scd_ssca(const void* x, int64_t N, int32_t Np, const float* window, void* out, const scd_opts* opts) {
-  scd::NvtxRange range("scd_ssca");
+}  // extern "C"
+
+namespace scd {
+scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, void* out, const scd_opts& o,
+                    const TuneEntry* given) {
   scd_status s = check_ssca(x, N, Np, window, out);
   if (s != SCD_OK) return s;
-  const scd_opts& o = opts_or_default(opts);
   if (o.precision != SCD_FP32 && o.precision != SCD_SPLIT_BF16) return SCD_ERR_UNSUPPORTED;
   if (!variant_ok(o)) return SCD_ERR_ARG;
   const float2* y = (const float2*)(o.y ? o.y : x);
@@ -195,12 +197,31 @@ scd_status scd_ssca(const void* x, int64_t N, int32_t Np, const float* window, v
     if ((e = m.mark(3, st)) != cudaSuccess) return cuda_fail(e);
     return SCD_OK;
   }
-  scd::TuneEntry choice{o.schedule, 0, 0, 0.0};
-  if (o.schedule == SCD_SCHEDULE_AUTO) choice = scd::ssca_auto_choice(N, Np, o.precision);
+  TuneEntry choice{o.schedule, 0, 0, 0.0};
+  const bool automatic = given || o.schedule == SCD_SCHEDULE_AUTO;
+  if (automatic) choice = given ? *given : scd::ssca_auto_choice(N, Np, o.precision);
   if (choice.schedule != SCD_SCHEDULE_STAGES && choice.schedule != SCD_SCHEDULE_PERSISTENT &&
       choice.schedule != SCD_SCHEDULE_FUSED)
     return SCD_ERR_ARG;
-  if (choice.schedule == SCD_SCHEDULE_FUSED && scd::ssca_fused_supported(N, Np, o.precision)) {
+  const bool fused = scd::ssca_fused_supported(N, Np, o.precision);
+  // the auto estimate under AUTO or FUSED: the lag-domain kernels (an explicit FUSED where its tiles
+  // do not fit asks for the STAGES kernels)
+  if (choice.schedule == SCD_SCHEDULE_FUSED && o.precision == SCD_FP32 && !o.y && !conj &&
+      (fused || automatic)) {
+    // events as the fused schedule records them (before, between the strip and the channel transforms,
+    // after); at the sizes where AUTO used to run STAGES, one more between the strip's two passes
+    StageMarks m{o, fused ? 3 : 4};
+    int mk = 0;
+    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_cols((const float2*)x, N, Np, ws, st)) != cudaSuccess) return cuda_fail(e);
+    if (!fused && (e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_rows(N, Np, ws, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_chan(ws, N, Np, window, (float2*)out, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
+    return SCD_OK;
+  }
+  if (choice.schedule == SCD_SCHEDULE_FUSED && fused) {
     StageMarks m{o, 3};
     if ((e = m.mark(0, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = scd::ssca_fused_chancol((const float2*)x, y, conj, N, Np, window, ws, st)) != cudaSuccess)
@@ -235,7 +256,13 @@ scd_status scd_ssca(const void* x, int64_t N, int32_t Np, const float* window, v
   return SCD_OK;
 }
 
-}  // extern "C"
+}  // namespace scd
+
+extern "C" scd_status scd_ssca(const void* x, int64_t N, int32_t Np, const float* window, void* out,
+                               const scd_opts* opts) {
+  scd::NvtxRange range("scd_ssca");
+  return scd::ssca_run(x, N, Np, window, out, opts_or_default(opts), nullptr);
+}
 
 namespace {
 scd_status check_fam_grid(const void* S, int32_t Np, int32_t L, int32_t P, const float* dst) {
@@ -336,6 +363,7 @@ scd_status scd_prepare(int32_t estimator, int64_t N, int32_t Np, int32_t P) {
     if (!scd::table_roots((int)M, &e) || !scd::table_pass(M1, &e) || !scd::table_pass(M2, &e) ||
         !scd::table_cols((int)M, M1, scd::ssca_cols_per_tile(M1), &e) || !scd::device_error_word(&e))
       return cuda_fail(e);
+    if (scd::is_pow2(N) && !scd::ssca_lag_tables(N, Np, &e)) return cuda_fail(e);
     if (!scd::is_pow2(N) && (!scd::table_chirp(N, &e) || !scd::table_bluestein_rows(N, M, M1, &e)))
       return cuda_fail(e);
     return SCD_OK;

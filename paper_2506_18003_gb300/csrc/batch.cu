@@ -25,7 +25,7 @@
 #include <vector>
 
 #include "batch_kernel.cuh"
-#include "ssca_fused.cuh"
+#include "ssca_lag.cuh"
 
 namespace scd {
 namespace bk {
@@ -332,13 +332,10 @@ scd_status build_tasks(scd_batch_plan* p) {
       p->st_launches.push_back(L);
       return SCD_OK;
     };
-    // fused SSCA kernels (staged == 2, FP32 form) for the size classes their tiles fit
-    const bool fused = !fam && !tc && p->staged == 2;
-    auto fused_n = [&](int64_t N, FusedSplit* fs) { return fused && fused_split(N, Np, fs); };
+    // staged == 2: the FP32 SSCA in the lag domain
+    const bool lag = !fam && !tc && p->staged == 2;
     int f0 = 0;
-    for (int i = 0; i < nsig; ++i) {
-      FusedSplit fs;
-      if (fused_n(p->sizes[i], &fs)) continue;                  // its channeliser runs inside tile A
+    for (int i = 0; i < nsig && !lag; ++i) {
       Task t = stage0_task(i);
       t.subtiles = t.tiles;
       p->st_tasks.push_back(t);
@@ -362,23 +359,25 @@ scd_status build_tasks(scd_batch_plan* p) {
       if ((ls = launch_of(p->prof_power ? 6 : 4, (int)P, f0)) != SCD_OK) return ls;
     }
     for (int64_t N : fam ? std::vector<int64_t>() : classes) {
-      FusedSplit fs;
-      if (fused_n(N, &fs)) {
-        // tile A (kind 7, clusters of fs.Q CTAs), then tile B (kind 8; 9 reduces into profiles)
-        for (int kind = 7; kind <= 8; ++kind) {
+      if (lag) {
+        // the three passes over every signal of the size (batch_lag.cu); launching them per group of
+        // signals whose intermediates fit L2 measured slower (512 signals: 15.37 ms whole classes,
+        // 15.43 groups of 64 MB, 15.98 of 32 MB)
+        LagSplit sp;
+        if (!lag_split(N, &sp)) return SCD_ERR_INTERNAL;
+        for (int kind = 7; kind <= 9; ++kind) {
+          const int M = kind == 7 ? sp.M1 : (kind == 8 ? sp.M2 : Np);
           f0 = (int)p->st_tasks.size();
           for (int i = 0; i < nsig; ++i) {
             if (p->sizes[i] != N) continue;
             Task t = stage0_task(i);
-            t.M1 = fs.M1; t.M2 = fs.M2;
-            t.size = kind == 7 ? fs.M1 : fs.M2;
-            t.subtiles = kind == 7 ? (int64_t)fs.M2 * fs.Q : (int64_t)Np * (fs.M1 / rowsf_c(fs.M2));
-            if (!(t.tw = table_pass(t.size, &e))) return cuda_status(e);
-            if (kind == 7 && !(t.wN = table_roots((int)N, &e))) return cuda_status(e);
+            t.M1 = sp.M1; t.M2 = sp.M2; t.size = M;
+            t.subtiles = kind == 7 ? lag_cols_tiles(Np, sp.M1, sp.M2)
+                                   : (kind == 8 ? lag_rows_tiles(Np, sp.M1, sp.M2) : lag_chan_tiles(Np, sp.M1, sp.M2));
+            if (!(t.tw = table_pass2(M, &e)) || !(t.wN = table_roots((int)N, &e))) return cuda_status(e);
             p->st_tasks.push_back(t);
           }
-          if ((ls = launch_of(kind == 8 && p->prof_power ? 9 : kind, kind == 7 ? (int)N : fs.M2, f0)) != SCD_OK)
-            return ls;
+          if ((ls = launch_of(kind, M, f0)) != SCD_OK) return ls;
         }
         continue;
       }
@@ -1134,8 +1133,7 @@ scd_status ssca_persistent(const float2* x, const float2* y, bool conj, int64_t 
 TuneEntry ssca_auto_choice(int64_t N, int Np, int precision) {
   TuneEntry e;
   if (tune_lookup(ssca_key(N, Np, precision), &e)) return e;
-  return TuneEntry{ssca_fused_supported(N, Np, precision) ? SCD_SCHEDULE_FUSED : SCD_SCHEDULE_STAGES, kItemBytes,
-                   kSlotBytes, 0.0};
+  return TuneEntry{precision == SCD_FP32 ? SCD_SCHEDULE_FUSED : SCD_SCHEDULE_STAGES, kItemBytes, kSlotBytes, 0.0};
 }
 
 void release_single_plans() {
@@ -1160,9 +1158,11 @@ extern "C" scd_status scd_ssca_tune(const void* x, int64_t N, int32_t Np, const 
   scd_status s = time_candidate(st, reps, [&]() { return scd_ssca(x, N, Np, window, out, &o); }, &ms);
   if (s != SCD_OK) return s;
   best.ms = ms;
-  if (ssca_fused_supported(N, Np, o.precision)) {
-    o.schedule = SCD_SCHEDULE_FUSED;
-    s = time_candidate(st, reps, [&]() { return scd_ssca(x, N, Np, window, out, &o); }, &ms);
+  if (o.precision == SCD_FP32 && is_pow2(N)) {
+    // what AUTO runs when never tuned: the lag-domain kernels, or the fused ones for a cross or
+    // conjugate estimate
+    const TuneEntry fused{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, 0.0};
+    s = time_candidate(st, reps, [&]() { return ssca_run(x, N, Np, window, out, o, &fused); }, &ms);
     if (s != SCD_OK) return s;
     if (ms < best.ms) best = TuneEntry{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, ms};
   }

@@ -17,6 +17,7 @@ namespace scd {
 // the first call for a size must not happen inside a stream capture.
 const float2* table_roots(int M, cudaError_t* err);        // W_M^j, j in [0, M)
 const float2* table_pass(int M, cudaError_t* err);         // Stockham pass twiddles of a size-M FFT
+const float2* table_pass2(int M, cudaError_t* err);        // ... of a paired size-M FFT (fft2.cuh)
 const float2* table_cols(int N, int M1, int C, cudaError_t* err);  // W_N^{c m1'}, [m1'][c], c < C
 const float* table_hamming(int Np, cudaError_t* err);      // default window, float32
 // Bluestein tables of a length-N DFT carried by size-M transforms (M a power of two >= 2N - 1):
@@ -73,6 +74,14 @@ cudaError_t ssca_fused_chancol(const float2* x, const float2* y, bool conj, int6
                                float2* ws, cudaStream_t st);
 cudaError_t ssca_fused_rows(const float2* ws, int64_t N, int Np, float2* out, cudaStream_t st);
 
+// Auto estimates in the lag domain (ssca_lag.cu, ssca_lag.cuh; FP32 form, N a power of two): cols =
+// lag products, M1-point pass and rotate factor into ws; rows = the M2-point pass in place on ws;
+// chan = window and Np-point transform over the lags into out[kh][sh].  ws: 8 (Np/2 + 2) N bytes.
+bool ssca_lag_tables(int64_t N, int Np, cudaError_t* err);      // builds the tables the three use
+cudaError_t ssca_lag_cols(const float2* x, int64_t N, int Np, float2* ws, cudaStream_t st);
+cudaError_t ssca_lag_rows(int64_t N, int Np, float2* ws, cudaStream_t st);
+cudaError_t ssca_lag_chan(const float2* ws, int64_t N, int Np, const float* window, float2* out, cudaStream_t st);
+
 // Default schedule of scd_ssca: one persistent launch (batch.cu) over a cached one-signal plan.
 size_t ssca_persistent_workspace(int64_t N, int Np);
 // y, conj: the channel-data product's second factor, as ssca_cdp
@@ -115,8 +124,11 @@ struct TuneEntry {
 std::string device_key();                                    // "<GPU name>/sm<cc>"
 bool tune_lookup(const std::string& key, TuneEntry* out);
 void tune_store(const std::string& key, const TuneEntry& e);
-// scd_ssca under SCD_SCHEDULE_AUTO: the tuned choice, else the default (STAGES)
+// scd_ssca under SCD_SCHEDULE_AUTO: the tuned choice, else the default (FUSED in the FP32 form)
 TuneEntry ssca_auto_choice(int64_t N, int Np, int precision);
+// scd_ssca with the choice AUTO makes given (NULL: from o.schedule, the tuned choice or the default)
+scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, void* out, const scd_opts& o,
+                    const TuneEntry* choice);
 scd_status ssca_persistent_tuned(const float2* x, const float2* y, bool conj, int64_t N, int Np, const float* window,
                                  float2* out, void* ws, size_t ws_bytes, cudaStream_t st, int precision,
                                  int64_t item_bytes, int64_t slot_bytes);

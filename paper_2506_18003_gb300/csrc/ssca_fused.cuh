@@ -212,30 +212,18 @@ __device__ __forceinline__ void ssca_chancol_tile(float2* sm, const float2* __re
 
 // Tile B: the q1 in [q10, q10 + C) of one channel, q10 a multiple of C: Yk = that channel's
 // row of Y (yf_index), outk = its output row (N values, fftshifted).
-// PROF: instead of storing S, every bin is reduced into the alpha profile prof[ah_off + sh]
-// (ah_off = k N/Np + N/2 for channel k) by profile_max of |S|^power (as ssca_rows_tile).
-template <int M2, bool PROF = false>
+template <int M2>
 __device__ __forceinline__ void ssca_rowsf_tile(float2* sm, const float2* __restrict__ Yk, float2* __restrict__ outk,
-                                                int M1, const float2* __restrict__ tw_m2, int q10,
-                                                float* prof = nullptr, int ah_off = 0, int power = 1) {
+                                                int M1, const float2* __restrict__ tw_m2, int q10) {
   using S = TileShape<M2, rowsf_threads(M2)>;
   constexpr int C = S::C;
   static_assert(C == rowsf_c(M2), "Y's column blocks are the second pass's tiles");
   const int c = (int)threadIdx.x % C;                   // interleaved: consecutive lanes, consecutive q1
   const float2* __restrict__ ib = Yk + (int64_t)q10 * M2 + c;
   auto src = [&](int, int m2) -> float2 { return ib[m2 * C]; };
-  if constexpr (PROF) {
-    unsigned* __restrict__ pr = reinterpret_cast<unsigned*>(prof) + ah_off + q10 + c;
-    auto dst = [&](int, int q2, float2 v) {
-      const float m2 = fmaf(v.x, v.x, v.y * v.y);
-      profile_max(pr + M1 * ((q2 + M2 / 2) & (M2 - 1)), __float_as_uint(power == 2 ? m2 : sqrtf(m2)));
-    };
-    fft_batch<M2, C, true, false>(sm, tw_m2, src, dst);
-  } else {
-    float2* __restrict__ ob = outk + q10 + c;
-    auto dst = [&](int, int q2, float2 v) { ob[(int64_t)M1 * ((q2 + M2 / 2) & (M2 - 1))] = v; };
-    fft_batch<M2, C, true, false>(sm, tw_m2, src, dst);
-  }
+  float2* __restrict__ ob = outk + q10 + c;
+  auto dst = [&](int, int q2, float2 v) { ob[(int64_t)M1 * ((q2 + M2 / 2) & (M2 - 1))] = v; };
+  fft_batch<M2, C, true, false>(sm, tw_m2, src, dst);
 }
 
 }  // namespace scd

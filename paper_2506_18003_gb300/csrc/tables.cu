@@ -16,6 +16,7 @@
 
 #include <cuda_bf16.h>
 
+#include "fft2.cuh"
 #include "fft_tc.cuh"
 #include "internal.h"
 
@@ -227,6 +228,21 @@ const float2* table_pass(int M, cudaError_t* err) {
   return (const float2*)get_or_build(1, M, 0, 0, sizeof(float2) * (size_t)len, err, [&](void* p, cudaStream_t st) {
     if (r.r1) k_pass<<<grid_for(len), 256, 0, st>>>((float2*)p, M, r.r0, r.r1, r.r2);
     else cudaMemsetAsync(p, 0, sizeof(float2), st);
+  });
+}
+
+// The paired transforms' table (Plan2's radices, same layout).
+const float2* table_pass2(int M, cudaError_t* err) {
+  PassRadices r{0, 0, 0};
+#define SCD_PR(MM) case MM: r = {Plan2<MM>::r[0], Plan2<MM>::r[1], Plan2<MM>::r[2]}; break;
+  switch (M) {
+    SCD_PR(16) SCD_PR(32) SCD_PR(64) SCD_PR(128) SCD_PR(256) SCD_PR(512) SCD_PR(1024)
+    default: *err = cudaErrorInvalidValue; return nullptr;
+  }
+#undef SCD_PR
+  const int len = pass_table_len(r.r0, r.r1, r.r2);
+  return (const float2*)get_or_build(11, M, 0, 0, sizeof(float2) * (size_t)len, err, [&](void* p, cudaStream_t st) {
+    k_pass<<<grid_for(len), 256, 0, st>>>((float2*)p, M, r.r0, r.r1, r.r2);
   });
 }
 
