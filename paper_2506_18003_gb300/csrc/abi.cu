@@ -213,9 +213,9 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
     StageMarks m{o, fused ? 3 : 4};
     int mk = 0;
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_cols((const float2*)x, N, Np, ws, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_strip((const float2*)x, N, Np, ws, (float2*)out, 0, st)) != cudaSuccess) return cuda_fail(e);
     if (!fused && (e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_rows(N, Np, ws, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_strip((const float2*)x, N, Np, ws, (float2*)out, 1, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = scd::ssca_lag_chan(ws, N, Np, window, (float2*)out, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);

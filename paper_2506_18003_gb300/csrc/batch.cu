@@ -97,6 +97,13 @@ struct scd_batch_plan {
   std::vector<scd::bk::Task> st_tasks;
   std::vector<StageLaunch> st_launches;
   scd::bk::Task* d_st = nullptr;
+  // lag-domain SSCA passes (ssca_lag.cuh) after the staged launches: kind 0 cols, 1 rows, 2 chan, over the
+  // signals lag_sigs[first ..], R of the first at r0 (the signals of one size are neighbours in the
+  // workspace); the arenas and the window are filled in per run
+  struct LagLaunch { int kind; int64_t first, r0; scd::LagArgs args; };
+  std::vector<scd::LagSig> lag_sigs;
+  std::vector<LagLaunch> lag_launches;
+  scd::LagSig* d_lag = nullptr;
   unsigned* d_counters = nullptr;
   int64_t total = 0;
   size_t ws_bytes = 0;
@@ -149,6 +156,7 @@ void free_plan(scd_batch_plan* p) {
   drop_graphs(p);
   if (p->d_tasks) cudaFree(p->d_tasks);
   if (p->d_st) cudaFree(p->d_st);
+  if (p->d_lag) cudaFree(p->d_lag);
   if (p->d_counters) cudaFree(p->d_counters);
   delete p;
 }
@@ -307,8 +315,11 @@ scd_status build_tasks(scd_batch_plan* p) {
   if (p->total >= (int64_t)0xFFFFFFF0u) return SCD_ERR_UNSUPPORTED;
   drop_graphs(p);
   if (p->d_st) { cudaFree(p->d_st); p->d_st = nullptr; }
+  if (p->d_lag) { cudaFree(p->d_lag); p->d_lag = nullptr; }
   p->st_tasks.clear();
   p->st_launches.clear();
+  p->lag_sigs.clear();
+  p->lag_launches.clear();
   if (p->staged) {
     // staged schedule: every signal's channeliser, then per size class (ascending N or P) the
     // SSCA column passes and row passes, or the FAM pair transforms, of its signals
@@ -360,25 +371,36 @@ scd_status build_tasks(scd_batch_plan* p) {
     }
     for (int64_t N : fam ? std::vector<int64_t>() : classes) {
       if (lag) {
-        // the three passes over every signal of the size (batch_lag.cu); launching them per group of
-        // signals whose intermediates fit L2 measured slower (512 signals: 15.37 ms whole classes,
-        // 15.43 groups of 64 MB, 15.98 of 32 MB)
+        // (passes over groups of signals whose intermediates fit L2 measured slower than over the
+        // whole class: 512 signals 15.37 ms, groups of 64 MB 15.43, of 32 MB 15.98)
         LagSplit sp;
         if (!lag_split(N, &sp)) return SCD_ERR_INTERNAL;
-        for (int kind = 7; kind <= 9; ++kind) {
-          const int M = kind == 7 ? sp.M1 : (kind == 8 ? sp.M2 : Np);
-          f0 = (int)p->st_tasks.size();
-          for (int i = 0; i < nsig; ++i) {
-            if (p->sizes[i] != N) continue;
-            Task t = stage0_task(i);
-            t.M1 = sp.M1; t.M2 = sp.M2; t.size = M;
-            t.subtiles = kind == 7 ? lag_cols_tiles(Np, sp.M1, sp.M2)
-                                   : (kind == 8 ? lag_rows_tiles(Np, sp.M1, sp.M2) : lag_chan_tiles(Np, sp.M1, sp.M2));
-            if (!(t.tw = table_pass2(M, &e)) || !(t.wN = table_roots((int)N, &e))) return cuda_status(e);
-            p->st_tasks.push_back(t);
-          }
-          if ((ls = launch_of(kind, M, f0)) != SCD_OK) return ls;
+        LagArgs A{};
+        A.N = (int)N; A.M1 = sp.M1; A.M2 = sp.M2; A.Np = Np; A.power = p->prof_power; A.err = p->err;
+        const int64_t first = (int64_t)p->lag_sigs.size();
+        int64_t r0 = -1;
+        for (int i = 0; i < nsig; ++i) {
+          if (p->sizes[i] != N) continue;
+          if (r0 < 0) r0 = p->ws_off[i];
+          // Y where S will be, or (profiles) behind R, which takes Np/2 + 1 of the signal's Np rows
+          p->lag_sigs.push_back({p->x_off[i], p->prof_power ? p->ws_off[i] + (Np / 2 + 1) * N : p->out_off[i],
+                                 p->ws_off[i], p->out_off[i]});
+          ++A.nsig;
         }
+        if (!(A.wN = table_roots((int)N, &e)) || (e = lag_prepare(sp.M1, sp.M2, Np)) != cudaSuccess) return cuda_status(e);
+        auto pass = [&](int kind, int M, int p0, int np) {
+          A.p0 = p0; A.np = np;
+          if (!(A.tw = table_pass2(M, &e))) return cuda_status(e);
+          p->lag_launches.push_back({kind, first, r0, A});
+          return SCD_OK;
+        };
+        // profiles: Y holds half of the lag pairs at a time (Np/2 - 1 rows are left for it)
+        const int pairs = lag_pairs(Np), group = p->prof_power ? (pairs + 1) / 2 : pairs;
+        for (int p0 = 0; p0 < pairs; p0 += group) {
+          const int np = std::min(group, pairs - p0);
+          if ((ls = pass(0, sp.M1, p0, np)) != SCD_OK || (ls = pass(1, sp.M2, p0, np)) != SCD_OK) return ls;
+        }
+        if ((ls = pass(2, Np, 0, pairs)) != SCD_OK) return ls;
         continue;
       }
       int M1, M2;
@@ -400,9 +422,15 @@ scd_status build_tasks(scd_batch_plan* p) {
         if ((ls = launch_of(kind == 2 && p->prof_power ? 5 : kind, M, f0)) != SCD_OK) return ls;
       }
     }
-    if ((e = cudaMalloc(&p->d_st, sizeof(Task) * p->st_tasks.size())) != cudaSuccess ||
-        (e = cudaMemcpy(p->d_st, p->st_tasks.data(), sizeof(Task) * p->st_tasks.size(), cudaMemcpyHostToDevice)) !=
-            cudaSuccess)
+    if (!p->st_tasks.empty() &&
+        ((e = cudaMalloc(&p->d_st, sizeof(Task) * p->st_tasks.size())) != cudaSuccess ||
+         (e = cudaMemcpy(p->d_st, p->st_tasks.data(), sizeof(Task) * p->st_tasks.size(), cudaMemcpyHostToDevice)) !=
+             cudaSuccess))
+      return cuda_status(e);
+    if (!p->lag_sigs.empty() &&
+        ((e = cudaMalloc(&p->d_lag, sizeof(LagSig) * p->lag_sigs.size())) != cudaSuccess ||
+         (e = cudaMemcpy(p->d_lag, p->lag_sigs.data(), sizeof(LagSig) * p->lag_sigs.size(), cudaMemcpyHostToDevice)) !=
+             cudaSuccess))
       return cuda_status(e);
   }
   if (p->d_tasks) { cudaFree(p->d_tasks); p->d_tasks = nullptr; }
@@ -478,7 +506,14 @@ scd_status plan_create(int32_t estimator, int32_t nsig, const int64_t* lengths, 
     p->used[i] = used;
     if (starts) p->x_off[i] = starts[i];
     p->x_off[i + 1] = starts ? span : p->x_off[i] + len;
-    p->ws_off[i + 1] = p->ws_off[i] + (int64_t)Np * sz;
+    p->ws_off[nsig] += (int64_t)Np * sz;
+  }
+  {                                                             // signals of one size side by side
+    std::vector<int> order(nsig);
+    for (int i = 0; i < nsig; ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return p->sizes[a] < p->sizes[b]; });
+    int64_t at = 0;
+    for (int i : order) { p->ws_off[i] = at; at += (int64_t)Np * p->sizes[i]; }
   }
   layout_outputs(p);
   // tables
@@ -835,7 +870,7 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   const size_t cbytes = sizeof(unsigned) * (p->tasks.size() + 1);
   // profiles are maxima of non-negative values: they start from 0 on every run
   const size_t pbytes = prof ? sizeof(float) * (size_t)p->out_off[p->nsig] : 0;
-  const bool staged = !p->st_launches.empty();
+  const bool staged = !p->st_launches.empty() || !p->lag_launches.empty();
   auto launch_all = [&]() -> cudaError_t {
     if (!staged) return launch_batch(fam, tc, prof, grid, p->smem, A, st);
     for (const auto& L : p->st_launches) {
@@ -843,9 +878,16 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
           staged_launch(L.kind, L.M, p->Np, tc, L.grid, L.smem, A, p->d_st + L.first, L.count, L.total, st);
       if (el != cudaSuccess) return el;
     }
+    for (const auto& L : p->lag_launches) {
+      LagArgs G = L.args;
+      G.sig = p->d_lag + L.first;
+      G.x = A.x; G.R = A.ws; G.Y = prof ? A.ws : A.out; G.out = A.out; G.prof = (float*)A.out; G.window = w;
+      const cudaError_t el = L.kind == 0 ? lag_cols(G, st) : (L.kind == 1 ? lag_rows(G, st) : lag_chan(G, L.r0, prof, st));
+      if (el != cudaSuccess) return el;
+    }
     return cudaSuccess;
   };
-  count_launches(staged ? (int)p->st_launches.size() : 1);
+  count_launches(staged ? (int)(p->st_launches.size() + p->lag_launches.size()) : 1);
   if (!st) {                                                    // legacy stream: no capture, plain launch
     if ((e = cudaMemsetAsync(p->d_counters, 0, cbytes, st)) != cudaSuccess) return cuda_status(e);
     if (prof && (e = cudaMemsetAsync(out_arena, 0, pbytes, st)) != cudaSuccess) return cuda_status(e);

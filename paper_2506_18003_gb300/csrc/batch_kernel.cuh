@@ -305,10 +305,6 @@ cudaError_t staged_launch(int kind, int M, int Np, bool tc, int grid, int smem, 
 // into the channel-data product's second factor, zero padding), 11 / 13 the two Bluestein
 // column passes (M = M1), 12 the fused middle pass (M = M2), 14 the FAM pair transform of any
 // P (M = the cyclic length MM).
-// Lag-domain SSCA passes (batch_lag.cu), kinds 7..9 of the staged schedule.
-cudaError_t lag_prepare(int kind, int M, int* smem);
-cudaError_t lag_launch(int kind, int M, int grid, int smem, const BatchArgs& A, const Task* tl, int nt,
-                       cudaStream_t st);
 cudaError_t exact_prepare(int kind, int M, int Np, bool tc, int* smem, int* per_sm);
 int exact_prep_per_tile();                                   // values of one signal per kind-10 CTA
 cudaError_t exact_launch(int kind, int M, int Np, bool tc, int grid, int smem, const BatchArgs& A, const Task* tl,

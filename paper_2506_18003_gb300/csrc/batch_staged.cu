@@ -216,8 +216,7 @@ void launch_m(int kind, int grid, int smem, const BatchArgs& A, const Task* tl, 
 
 // kinds: SSCA 0 channeliser + CDP (M = Np in 16..256), 1 column pass (M = M1), 2 row pass
 // (M = M2), M1 and M2 in 64..1024; FAM 3 channeliser (M = Np), 4 pair transforms (M = P in
-// 2..8192); 5 and 6: kinds 2 and 4 reducing into alpha profiles; 7, 8, 9: the lag-domain SSCA
-// passes (batch_lag.cu, FP32 form)
+// 2..8192); 5 and 6: kinds 2 and 4 reducing into alpha profiles
 bool valid(int kind, int M, bool tc) {
   const bool pow2 = M >= 2 && (M & (M - 1)) == 0;
   if (kind == 0 || kind == 3) return pow2 && M >= 16 && M <= 256;
@@ -229,7 +228,6 @@ bool valid(int kind, int M, bool tc) {
 
 cudaError_t staged_prepare(int kind, int M, int Np, bool tc, int* smem, int* per_sm) {
   if (kind >= 10) return exact_prepare(kind, M, Np, tc, smem, per_sm);
-  if (kind >= 7) return tc ? cudaErrorInvalidValue : lag_prepare(kind, M, smem);
   if (!valid(kind, M, tc)) return cudaErrorInvalidValue;
 #define SCD_SP(MV) case MV: return tc ? prep_m<MV, true>(kind, smem, per_sm) : prep_m<MV, false>(kind, smem, per_sm);
   switch (M) {
@@ -243,7 +241,6 @@ cudaError_t staged_prepare(int kind, int M, int Np, bool tc, int* smem, int* per
 cudaError_t staged_launch(int kind, int M, int Np, bool tc, int grid, int smem, const BatchArgs& A, const Task* tl,
                           int nt, int64_t total, cudaStream_t st) {
   if (kind >= 10) return exact_launch(kind, M, Np, tc, grid, smem, A, tl, nt, total, st);
-  if (kind >= 7) return tc ? cudaErrorInvalidValue : lag_launch(kind, M, grid, smem, A, tl, nt, st);
   if (!valid(kind, M, tc)) return cudaErrorInvalidValue;
 #define SCD_SL(MV) case MV: if (tc) launch_m<MV, true>(kind, grid, smem, A, tl, nt, total, st); else launch_m<MV, false>(kind, grid, smem, A, tl, nt, total, st); break;
   switch (M) {

@@ -17,33 +17,18 @@
 // Per tile (columns m2 = m20 + c of channel kh): M1-point DFT over m1, times the rotate factor
 // W_N^{(m2 m1') mod N} (split as in ssca_cols_tile), written in place to Y[kh][m1'][m2] (the
 // tile's own input, already in shared memory).
-#include <cuda.h>
 #include <cudaTypedefs.h>
 
 #include <mutex>
 
 #include "internal.h"
-#include "tiles.cuh"
+#include "tma.cuh"
 
 namespace scd {
 namespace {
 
 // Bounded waits: every poll loop gives up after this many polls.
 constexpr uint32_t kTmaPollLimit = kMbarPollLimit;
-
-__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(su32(mbar)), "r"(bytes) : "memory");
-}
-
-// One box of the 3-D tensor map into shared memory; x is the innermost coordinate (m2).
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      :: "r"(su32(dst)), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(su32(mbar))
-      : "memory");
-}
 
 template <int M1>
 struct ColsTma {
@@ -136,7 +121,37 @@ k_ssca_cols_tma(const __grid_constant__ CUtensorMap tm, float2* __restrict__ Y, 
   if (tid == 0) umma::mbar_inval(mbar);
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn(cudaError_t* err) {
+template <int M1>
+cudaError_t launch_t(float2* Y, int N, int Np, int M2, cudaStream_t st) {
+  using K = ColsTma<M1>;
+  cudaError_t e;
+  const float2* wN = table_roots(N, &e);
+  if (!wN) return e;
+  const float2* tw = table_pass(M1, &e);
+  if (!tw) return e;
+  unsigned* errw = device_error_word(&e);
+  if (!errw) return e;
+  // X_g as [Np][M1][M2] 8-byte elements (complex64 moved as raw 64-bit words)
+  CUtensorMap tm;
+  const cuuint64_t dims[3] = {(cuuint64_t)M2, (cuuint64_t)M1, (cuuint64_t)Np};
+  const cuuint64_t strides[2] = {(cuuint64_t)M2 * 8, (cuuint64_t)M1 * M2 * 8};
+  const cuuint32_t box[3] = {(cuuint32_t)K::C, (cuuint32_t)K::ROWS, 1};
+  if ((e = encode_map_c64(&tm, Y, 3, dims, strides, box)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_ssca_cols_tma<M1>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM)) !=
+      cudaSuccess)
+    return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int64_t ntiles = (int64_t)Np * (M2 / K::C);
+  const int grid = (int)(ntiles < 2 * sms ? ntiles : 2 * sms);         // two persistent CTAs per SM
+  k_ssca_cols_tma<M1><<<grid, 256, K::SMEM, st>>>(tm, Y, N, M2, Np, wN, tw, errw);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+static PFN_cuTensorMapEncodeTiled_v12000 encode_fn(cudaError_t* err) {
   static std::once_flag once;
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static cudaError_t status = cudaSuccess;
@@ -151,41 +166,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn(cudaError_t* err) {
   return fn;
 }
 
-template <int M1>
-cudaError_t launch_t(float2* Y, int N, int Np, int M2, cudaStream_t st) {
-  using K = ColsTma<M1>;
+cudaError_t encode_map_c64(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims,
+                           const cuuint64_t* strides, const cuuint32_t* box) {
   cudaError_t e;
   PFN_cuTensorMapEncodeTiled_v12000 encode = encode_fn(&e);
   if (!encode) return e;
-  const float2* wN = table_roots(N, &e);
-  if (!wN) return e;
-  const float2* tw = table_pass(M1, &e);
-  if (!tw) return e;
-  unsigned* errw = device_error_word(&e);
-  if (!errw) return e;
-  // X_g as [Np][M1][M2] 8-byte elements (complex64 moved as raw 64-bit words)
-  CUtensorMap tm;
-  const cuuint64_t dims[3] = {(cuuint64_t)M2, (cuuint64_t)M1, (cuuint64_t)Np};
-  const cuuint64_t strides[2] = {(cuuint64_t)M2 * 8, (cuuint64_t)M1 * M2 * 8};
-  const cuuint32_t box[3] = {(cuuint32_t)K::C, (cuuint32_t)K::ROWS, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  if (encode(&tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, Y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  if ((e = cudaFuncSetAttribute(k_ssca_cols_tma<M1>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM)) !=
-      cudaSuccess)
-    return e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int64_t ntiles = (int64_t)Np * (M2 / K::C);
-  const int grid = (int)(ntiles < 2 * sms ? ntiles : 2 * sms);         // two persistent CTAs per SM
-  k_ssca_cols_tma<M1><<<grid, 256, K::SMEM, st>>>(tm, Y, N, M2, Np, wN, tw, errw);
-  return cudaGetLastError();
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess
+             : cudaErrorInvalidValue;
 }
-
-}  // namespace
 
 bool ssca_cols_tma_supported(int M1) { return M1 == 1024; }
 

@@ -196,8 +196,9 @@ struct PairFft {
     return c2_from(*p);
 #endif
   }
+  // Twiddled inputs of pass S (tw: the pass table, in shared memory) and its radix transforms.
   template <int S>
-  __device__ __forceinline__ static void load(const float4* sm, const float2* __restrict__ tw, int c, int t, C2* v) {
+  __device__ __forceinline__ static void load(const float4* sm, const float2* tw, int c, int t, C2* v) {
     constexpr int R = PI::R(S), p = PI::p(S), B = E / R;
 #pragma unroll
     for (int b = 0; b < B; ++b) {
@@ -205,14 +206,20 @@ struct PairFft {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         C2 x = take(sm + at(c, i + r * (M / R)));
-        if (r > 0) x = cmul(x, __ldg(tw + PI::off(S) + r * p + k));
+        if (r > 0) x = cmul(x, tw[PI::off(S) + r * p + k]);
         v[b * R + r] = x;
       }
-      dft2<R>(v + b * R);
     }
   }
-  template <class Dst>
-  __device__ __forceinline__ static void run(float4* sm, const float2* __restrict__ tw, C2* v, Dst& dst) {
+  template <int S>
+  __device__ __forceinline__ static void dfts(C2* v) {
+    constexpr int R = PI::R(S), B = E / R;
+#pragma unroll
+    for (int b = 0; b < B; ++b) dft2<R>(v + b * R);
+  }
+  // free(): called when this thread has read the last of the exchange area
+  template <class Free, class Dst>
+  __device__ __forceinline__ static void run(float4* sm, const float2* tw, C2* v, Free&& free, Dst& dst) {
     constexpr int L = PI::n - 1, RL = PI::rl;
     const int c = in_c(), t = in_t(), co = out_c(), to = out_t();
     dft2<PI::r0>(v);
@@ -221,6 +228,7 @@ struct PairFft {
     if constexpr (PI::n == 3) {
       sync<false>();
       load<1>(sm, tw, c, t, v);
+      dfts<1>(v);
       sync<false>();                                       // every read of pass 1 precedes its writes
       constexpr int R = PI::r1, p = PI::r0;
 #pragma unroll
@@ -232,6 +240,8 @@ struct PairFft {
     }
     sync<true>();
     load<L>(sm, tw, co, to, v);
+    free();
+    dfts<L>(v);
 #pragma unroll
     for (int b = 0; b < E / RL; ++b)
 #pragma unroll

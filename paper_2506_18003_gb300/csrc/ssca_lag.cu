@@ -1,5 +1,5 @@
-// SSCA auto estimates in the lag domain, single estimates: the three passes of ssca_lag.cuh, one
-// kernel each.
+// SSCA auto estimates in the lag domain: the kernels of ssca_lag.cuh's three passes, for one signal or
+// for the signals of one size of a batch plan.
 #include "internal.h"
 #include "ssca_lag.cuh"
 
@@ -7,111 +7,179 @@ namespace scd {
 namespace {
 
 template <int M1>
-__global__ void __launch_bounds__(LagCols<M1>::NT, lag_strip_minb(M1))
-k_lag_cols(const float2* __restrict__ x, int N, int M2, const float2* __restrict__ tw, const float2* __restrict__ wN,
-           float4* __restrict__ Y) {
+__global__ void __launch_bounds__(LagCols<M1>::NT, LagCols<M1>::minb) k_lag_cols(const LagArgs A) {
   extern __shared__ __align__(128) unsigned char lag_sm[];
-  lag_cols_tile<M1>(lag_sm, x, N, M2, tw, wN, Y, (int)blockIdx.x);
+  lag_cols_tile<M1>(lag_sm, A, (int)blockIdx.x);
 }
-
 template <int M2>
-__global__ void __launch_bounds__(LagRows<M2>::NT, lag_strip_minb(M2))
-k_lag_rows(float4* __restrict__ Y, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(LagRows<M2>::NT, LagRows<M2>::minb) k_lag_rows(const LagArgs A) {
   extern __shared__ __align__(128) unsigned char lag_sm[];
-  lag_rows_tile<M2>(lag_sm, Y, tw, (int)blockIdx.x);
+  lag_rows_cta<M2>(lag_sm, A);
 }
-
-template <int NP>
-__global__ void __launch_bounds__(LagChan<NP>::NT, lag_chan_minb(NP))
-k_lag_chan(const float2* __restrict__ R, int N, int M1, int M2, const float* __restrict__ a,
-           const float2* __restrict__ tw, const float2* __restrict__ wN, float2* __restrict__ out) {
+template <int NP, int NTHR, bool PROF>
+__global__ void __launch_bounds__(NTHR, LagChan<NP, NTHR>::minb)
+k_lag_chan(const LagArgs A, const __grid_constant__ CUtensorMap tp, const __grid_constant__ CUtensorMap tn) {
   extern __shared__ __align__(128) unsigned char lag_sm[];
-  lag_chan_tile<NP, false>(lag_sm, R, N, M1, M2, a, tw, wN, out, (int)blockIdx.x);
+  lag_chan_cta<NP, NTHR, PROF>(lag_sm, A, &tp, &tn);
 }
 
 template <class K>
 cudaError_t set_smem(K kernel, int bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-template <int M1>
-cudaError_t launch_cols(const float2* x, int N, int Np, int M2, const float2* wN, float4* Y, cudaStream_t st) {
+// persistent CTAs of a launch over `tiles` tiles: per_sm of nt threads on every SM, of a large output at
+// most 512 threads
+cudaError_t grid_of(const LagArgs& A, int64_t tiles, int per_sm, int nt, unsigned* grid) {
+  if (lag_large(A.N, A.Np, A.nsig) && per_sm * nt > 512) per_sm = 512 / nt;
+  int dev = 0, sms = 0;
   cudaError_t e;
-  const float2* tw = table_pass2(M1, &e);
-  if (!tw || (e = set_smem(k_lag_cols<M1>, LagCols<M1>::smem)) != cudaSuccess) return e;
-  k_lag_cols<M1><<<(unsigned)lag_cols_tiles(Np, M1, M2), LagCols<M1>::NT, LagCols<M1>::smem, st>>>(x, N, M2, tw, wN, Y);
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  *grid = (unsigned)(tiles < (int64_t)per_sm * sms ? tiles : (int64_t)per_sm * sms);
+  return cudaSuccess;
+}
+
+#define SCD_LAG_STRIP(X) X(64) X(128) X(256) X(512) X(1024)
+
+template <int M1>
+cudaError_t launch_cols(const LagArgs& A, cudaStream_t st) {
+  const int64_t tiles = (int64_t)lag_cols_tiles(A.np, M1, A.M2) * A.nsig;
+  if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
+  k_lag_cols<M1><<<(unsigned)tiles, LagCols<M1>::NT, LagCols<M1>::smem, st>>>(A);
   return cudaGetLastError();
 }
 
 template <int M2>
-cudaError_t launch_rows(int Np, int M1, float4* Y, cudaStream_t st) {
-  cudaError_t e;
-  const float2* tw = table_pass2(M2, &e);
-  if (!tw || (e = set_smem(k_lag_rows<M2>, LagRows<M2>::smem)) != cudaSuccess) return e;
-  k_lag_rows<M2><<<(unsigned)lag_rows_tiles(Np, M1, M2), LagRows<M2>::NT, LagRows<M2>::smem, st>>>(Y, tw);
+cudaError_t launch_rows(const LagArgs& A, cudaStream_t st) {
+  using K = LagRows<M2>;
+  const int64_t tiles = (int64_t)lag_rows_tiles(A.np, A.M1, M2) * A.nsig;
+  if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
+  unsigned grid;
+  cudaError_t e = grid_of(A, tiles, K::minb, K::NT, &grid);
+  if (e != cudaSuccess) return e;
+  k_lag_rows<M2><<<grid, K::NT, K::smem, st>>>(A);
   return cudaGetLastError();
 }
 
-template <int NP>
-cudaError_t launch_chan(const float2* R, int N, int M1, int M2, const float* a, const float2* wN, float2* out,
-                        cudaStream_t st) {
-  cudaError_t e;
-  const float2* tw = table_pass2(NP, &e);
-  if (!tw || (e = set_smem(k_lag_chan<NP>, LagChan<NP>::smem)) != cudaSuccess) return e;
-  k_lag_chan<NP><<<(unsigned)lag_chan_tiles(NP, M1, M2), LagChan<NP>::NT, LagChan<NP>::smem, st>>>(R, N, M1, M2, a, tw,
-                                                                                                 wN, out);
+template <int NP, int NTHR>
+cudaError_t launch_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st) {
+  using K = LagChan<NP, NTHR>;
+  const int64_t tiles = (int64_t)(A.N / (2 * K::C)) * A.nsig;
+  if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
+  unsigned grid;
+  cudaError_t e = grid_of(A, tiles, K::minb, K::NT, &grid);
+  if (e != cudaSuccess) return e;
+  CUtensorMap tp, tn;                                       // R as [signal][lag][c]
+  const cuuint64_t dims[3] = {(cuuint64_t)A.N, NP / 2 + 1, (cuuint64_t)A.nsig};
+  const cuuint64_t strides[2] = {(cuuint64_t)A.N * 8, (cuuint64_t)A.N * NP * 8};
+  const cuuint32_t bp[3] = {K::pos_row, NP / 2, 1}, bn[3] = {K::neg_row, NP / 2, 1};
+  if ((e = encode_map_c64(&tp, A.R + r0, 3, dims, strides, bp)) != cudaSuccess) return e;
+  if ((e = encode_map_c64(&tn, A.R + r0, 3, dims, strides, bn)) != cudaSuccess) return e;
+  if (prof) k_lag_chan<NP, NTHR, true><<<grid, K::NT, K::smem, st>>>(A, tp, tn);
+  else k_lag_chan<NP, NTHR, false><<<grid, K::NT, K::smem, st>>>(A, tp, tn);
   return cudaGetLastError();
 }
 
 }  // namespace
 
+cudaError_t lag_prepare(int M1, int M2, int Np) {
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (M1) {
+#define SCD_X(M) case M: e = set_smem(k_lag_cols<M>, LagCols<M>::smem); break;
+    SCD_LAG_STRIP(SCD_X)
+#undef SCD_X
+  }
+  if (e != cudaSuccess) return e;
+  e = cudaErrorInvalidValue;
+  switch (M2) {
+#define SCD_X(M) case M: e = set_smem(k_lag_rows<M>, LagRows<M>::smem); break;
+    SCD_LAG_STRIP(SCD_X)
+#undef SCD_X
+  }
+  if (e != cudaSuccess) return e;
+  e = cudaErrorInvalidValue;
+  switch (Np) {
+#define SCD_X(M, T)                                                                                \
+  if (e == cudaSuccess) e = set_smem(k_lag_chan<M, T, false>, LagChan<M, T>::smem);               \
+  if (e == cudaSuccess) e = set_smem(k_lag_chan<M, T, true>, LagChan<M, T>::smem);
+    case 16: e = cudaSuccess; SCD_X(16, 128) break;
+    case 32: e = cudaSuccess; SCD_X(32, 128) break;
+    case 64: e = cudaSuccess; SCD_X(64, 128) break;
+    case 128: e = cudaSuccess; SCD_X(128, 128) break;
+    case 256: e = cudaSuccess; SCD_X(256, 128) SCD_X(256, 256) break;
+#undef SCD_X
+  }
+  return e;
+}
+
+cudaError_t lag_cols(const LagArgs& A, cudaStream_t st) {
+  switch (A.M1) {
+#define SCD_X(M) case M: return launch_cols<M>(A, st);
+    SCD_LAG_STRIP(SCD_X)
+#undef SCD_X
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t lag_rows(const LagArgs& A, cudaStream_t st) {
+  switch (A.M2) {
+#define SCD_X(M) case M: return launch_rows<M>(A, st);
+    SCD_LAG_STRIP(SCD_X)
+#undef SCD_X
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t lag_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st) {
+  switch (A.Np) {
+    case 16: return launch_chan<16, 128>(A, r0, prof, st);
+    case 32: return launch_chan<32, 128>(A, r0, prof, st);
+    case 64: return launch_chan<64, 128>(A, r0, prof, st);
+    case 128: return launch_chan<128, 128>(A, r0, prof, st);
+    case 256:
+      return lag_large(A.N, 256, A.nsig) ? launch_chan<256, 256>(A, r0, prof, st) : launch_chan<256, 128>(A, r0, prof, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 bool ssca_lag_tables(int64_t N, int Np, cudaError_t* err) {
   LagSplit s;
   if (!lag_split(N, &s)) { *err = cudaErrorInvalidValue; return false; }
-  return table_pass2(s.M1, err) && table_pass2(s.M2, err) && table_pass2(Np, err) && table_roots((int)N, err);
+  return table_pass2(s.M1, err) && table_pass2(s.M2, err) && table_pass2(Np, err) && table_roots((int)N, err) &&
+         device_error_word(err);
 }
 
-cudaError_t ssca_lag_cols(const float2* x, int64_t N, int Np, float2* ws, cudaStream_t st) {
+namespace {
+// One signal: Y in the output's memory, R in the workspace.
+cudaError_t one(const float2* x, int64_t N, int Np, const float* window, float2* ws, float2* out, LagArgs* A) {
   LagSplit s;
   if (!lag_split(N, &s)) return cudaErrorInvalidValue;
+  *A = LagArgs{};
+  A->x = x; A->Y = out; A->R = ws; A->out = out; A->window = window;
+  A->N = (int)N; A->M1 = s.M1; A->M2 = s.M2; A->nsig = 1; A->Np = Np; A->np = lag_pairs(Np);
   cudaError_t e;
-  const float2* wN = table_roots((int)N, &e);
-  if (!wN) return e;
-  count_launches(1);
-  switch (s.M1) {
-#define SCD_LC(M) case M: return launch_cols<M>(x, (int)N, Np, s.M2, wN, (float4*)ws, st);
-    SCD_LC(64) SCD_LC(128) SCD_LC(256) SCD_LC(512) SCD_LC(1024)
-#undef SCD_LC
-    default: return cudaErrorInvalidValue;
-  }
+  if (!(A->wN = table_roots((int)N, &e)) || !(A->err = device_error_word(&e))) return e;
+  return lag_prepare(s.M1, s.M2, Np);
 }
+}  // namespace
 
-cudaError_t ssca_lag_rows(int64_t N, int Np, float2* ws, cudaStream_t st) {
-  LagSplit s;
-  if (!lag_split(N, &s)) return cudaErrorInvalidValue;
+cudaError_t ssca_lag_strip(const float2* x, int64_t N, int Np, float2* ws, float2* out, int pass, cudaStream_t st) {
+  LagArgs A;
+  cudaError_t e = one(x, N, Np, nullptr, ws, out, &A);
+  if (e != cudaSuccess) return e;
+  if (!(A.tw = table_pass2(pass == 0 ? A.M1 : A.M2, &e))) return e;
   count_launches(1);
-  switch (s.M2) {
-#define SCD_LR(M) case M: return launch_rows<M>(Np, s.M1, (float4*)ws, st);
-    SCD_LR(64) SCD_LR(128) SCD_LR(256) SCD_LR(512) SCD_LR(1024)
-#undef SCD_LR
-    default: return cudaErrorInvalidValue;
-  }
+  return pass == 0 ? lag_cols(A, st) : lag_rows(A, st);
 }
 
 cudaError_t ssca_lag_chan(const float2* ws, int64_t N, int Np, const float* window, float2* out, cudaStream_t st) {
-  LagSplit s;
-  if (!lag_split(N, &s)) return cudaErrorInvalidValue;
-  cudaError_t e;
-  const float2* wN = table_roots((int)N, &e);
-  if (!wN) return e;
+  LagArgs A;
+  cudaError_t e = one(nullptr, N, Np, window, const_cast<float2*>(ws), out, &A);
+  if (e != cudaSuccess) return e;
+  if (!(A.tw = table_pass2(Np, &e))) return e;
   count_launches(1);
-  switch (Np) {
-#define SCD_LN(M) case M: return launch_chan<M>(ws, (int)N, s.M1, s.M2, window, wN, out, st);
-    SCD_LN(16) SCD_LN(32) SCD_LN(64) SCD_LN(128) SCD_LN(256)
-#undef SCD_LN
-    default: return cudaErrorInvalidValue;
-  }
+  return lag_chan(A, 0, false, st);
 }
 
 }  // namespace scd
