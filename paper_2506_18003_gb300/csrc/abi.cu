@@ -349,7 +349,9 @@ scd_status scd_prepare(int32_t estimator, int64_t N, int32_t Np, int32_t P) {
   if (!scd::table_hamming(Np, &e) || !scd::table_roots(Np, &e) || !scd::table_pass(Np, &e)) return cuda_fail(e);
   if (estimator == 0) {
     if (P < 2 || P > 16384 || (!scd::is_pow2(P) && P > kMaxAnyP)) return SCD_ERR_UNSUPPORTED;
-    if (scd::is_pow2(P)) return scd::table_pass(P, &e) ? SCD_OK : cuda_fail(e);
+    if (scd::is_pow2(P)) {
+      return scd::table_pass(P, &e) && scd::fam_pair_tables(P, &e) ? SCD_OK : cuda_fail(e);
+    }
     const int64_t M = scd::bluestein_len_host(P);
     if (!scd::table_pass((int)M, &e) || !scd::table_chirp(P, &e) || !scd::table_bluestein(P, M, &e))
       return cuda_fail(e);

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "batch_kernel.cuh"
+#include "fam2.cuh"
 #include "ssca_lag.cuh"
 
 namespace scd {
@@ -97,7 +98,12 @@ struct scd_batch_plan {
   std::vector<scd::bk::Task> st_tasks;
   std::vector<StageLaunch> st_launches;
   scd::bk::Task* d_st = nullptr;
-  // lag-domain SSCA passes (ssca_lag.cuh) after the staged launches: kind 0 cols, 1 rows, 2 chan, over the
+  // FAM pair transforms of one size P over the signals fam_sigs[first ..] (fam2.cuh)
+  struct FamLaunch { int P; int64_t first; scd::FamArgs args; };
+  std::vector<scd::FamSig> fam_sigs;
+  std::vector<FamLaunch> fam_launches;
+  scd::FamSig* d_fam = nullptr;
+  // After the staged launches: lag-domain SSCA passes (ssca_lag.cuh): kind 0 cols, 1 rows, 2 chan, over the
   // signals lag_sigs[first ..], R of the first at r0 (the signals of one size are neighbours in the
   // workspace); the arenas and the window are filled in per run
   struct LagLaunch { int kind; int64_t first, r0; scd::LagArgs args; };
@@ -157,6 +163,7 @@ void free_plan(scd_batch_plan* p) {
   if (p->d_tasks) cudaFree(p->d_tasks);
   if (p->d_st) cudaFree(p->d_st);
   if (p->d_lag) cudaFree(p->d_lag);
+  if (p->d_fam) cudaFree(p->d_fam);
   if (p->d_counters) cudaFree(p->d_counters);
   delete p;
 }
@@ -168,12 +175,13 @@ scd_status cuda_status(cudaError_t e) {
   return SCD_ERR_CUDA;
 }
 
-// Schedule of a new plan's full estimates (the plan's `staged`: 0 persistent, 1 staged, 2 staged
-// with the fused SSCA kernels where their tiles fit): SSCA defaults to the staged schedule
-// (measured faster on every batch tried: 512 signals of 2^12..2^18 samples, Np = 128: 29.0 ->
-// 23.5 ms FP32, 42.0 -> 35.9 ms split), fused in the FP32 form; FAM to the persistent one.
+// Schedule of a new plan's full estimates (the plan's `staged`: 0 persistent, 1 staged, 2 staged with
+// the paired transforms: SSCA in the lag domain, FAM with fam2.cuh's pair kernels where they are the
+// faster ones).  FP32 plans default to 2: 512 signals of 2^12..2^18 samples, SSCA (Np = 128) persistent
+// 29.0 ms, staged 23.5, lag domain 12.8; FAM (Np = 64) persistent 12.6, staged 10.6, paired 10.5.  The
+// split form: SSCA staged (42.0 -> 35.9 ms), FAM persistent (17.3 against 19.9 ms staged).
 int default_staged(int estimator, int precision) {
-  return estimator == 1 ? (precision == SCD_FP32 ? 2 : 1) : 0;
+  return precision == SCD_FP32 ? 2 : (estimator == 1 ? 1 : 0);
 }
 
 // Output arena layout of the plan's mode: full estimates (complex64 elements: FAM Np^2 P_i,
@@ -316,10 +324,13 @@ scd_status build_tasks(scd_batch_plan* p) {
   drop_graphs(p);
   if (p->d_st) { cudaFree(p->d_st); p->d_st = nullptr; }
   if (p->d_lag) { cudaFree(p->d_lag); p->d_lag = nullptr; }
+  if (p->d_fam) { cudaFree(p->d_fam); p->d_fam = nullptr; }
   p->st_tasks.clear();
   p->st_launches.clear();
   p->lag_sigs.clear();
   p->lag_launches.clear();
+  p->fam_sigs.clear();
+  p->fam_launches.clear();
   if (p->staged) {
     // staged schedule: every signal's channeliser, then per size class (ascending N or P) the
     // SSCA column passes and row passes, or the FAM pair transforms, of its signals
@@ -357,6 +368,21 @@ scd_status build_tasks(scd_batch_plan* p) {
     std::sort(classes.begin(), classes.end());
     classes.erase(std::unique(classes.begin(), classes.end()), classes.end());
     for (int64_t P : fam ? classes : std::vector<int64_t>()) {
+      if (!tc && p->staged == 2 && fam2_supported((int)P, true)) {
+        FamArgs A{};
+        A.Np = Np; A.power = p->prof_power; A.PL = (int)P * p->L; A.Q = A.PL / Np;
+        const int64_t first = (int64_t)p->fam_sigs.size();
+        for (int i = 0; i < nsig; ++i) {
+          if (p->sizes[i] != P) continue;
+          p->fam_sigs.push_back({p->ws_off[i], p->out_off[i]});
+          ++A.nsig;
+        }
+        if (!(A.tw = table_pass2((int)P / 2, &e)) || !(A.wP = table_roots((int)P, &e)) ||
+            (e = fam2_prepare((int)P)) != cudaSuccess)
+          return cuda_status(e);
+        p->fam_launches.push_back({(int)P, first, A});
+        continue;
+      }
       f0 = (int)p->st_tasks.size();
       for (int i = 0; i < nsig; ++i) {
         if (p->sizes[i] != P) continue;
@@ -430,6 +456,11 @@ scd_status build_tasks(scd_batch_plan* p) {
     if (!p->lag_sigs.empty() &&
         ((e = cudaMalloc(&p->d_lag, sizeof(LagSig) * p->lag_sigs.size())) != cudaSuccess ||
          (e = cudaMemcpy(p->d_lag, p->lag_sigs.data(), sizeof(LagSig) * p->lag_sigs.size(), cudaMemcpyHostToDevice)) !=
+             cudaSuccess))
+      return cuda_status(e);
+    if (!p->fam_sigs.empty() &&
+        ((e = cudaMalloc(&p->d_fam, sizeof(FamSig) * p->fam_sigs.size())) != cudaSuccess ||
+         (e = cudaMemcpy(p->d_fam, p->fam_sigs.data(), sizeof(FamSig) * p->fam_sigs.size(), cudaMemcpyHostToDevice)) !=
              cudaSuccess))
       return cuda_status(e);
   }
@@ -870,12 +901,22 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   const size_t cbytes = sizeof(unsigned) * (p->tasks.size() + 1);
   // profiles are maxima of non-negative values: they start from 0 on every run
   const size_t pbytes = prof ? sizeof(float) * (size_t)p->out_off[p->nsig] : 0;
-  const bool staged = !p->st_launches.empty() || !p->lag_launches.empty();
+  // An injected drop is about the persistent launch's waits: a FAM plan on its default schedule runs that
+  // launch for it (as its default schedule used to).
+  const bool injected = A.drop_task >= 0 && fam && p->staged == 2;
+  const bool staged = !injected && (!p->st_launches.empty() || !p->lag_launches.empty());   // (FAM: the channeliser)
   auto launch_all = [&]() -> cudaError_t {
     if (!staged) return launch_batch(fam, tc, prof, grid, p->smem, A, st);
     for (const auto& L : p->st_launches) {
       cudaError_t el =
           staged_launch(L.kind, L.M, p->Np, tc, L.grid, L.smem, A, p->d_st + L.first, L.count, L.total, st);
+      if (el != cudaSuccess) return el;
+    }
+    for (const auto& L : p->fam_launches) {
+      FamArgs G = L.args;
+      G.sig = p->d_fam + L.first;
+      G.X = G.Y = A.ws; G.out = A.out; G.prof = (float*)A.out;
+      const cudaError_t el = fam2_pairs(G, L.P, true, prof, st);
       if (el != cudaSuccess) return el;
     }
     for (const auto& L : p->lag_launches) {
@@ -887,7 +928,7 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
     }
     return cudaSuccess;
   };
-  count_launches(staged ? (int)(p->st_launches.size() + p->lag_launches.size()) : 1);
+  count_launches(staged ? (int)(p->st_launches.size() + p->lag_launches.size() + p->fam_launches.size()) : 1);
   if (!st) {                                                    // legacy stream: no capture, plain launch
     if ((e = cudaMemsetAsync(p->d_counters, 0, cbytes, st)) != cudaSuccess) return cuda_status(e);
     if (prof && (e = cudaMemsetAsync(out_arena, 0, pbytes, st)) != cudaSuccess) return cuda_status(e);
@@ -1073,7 +1114,7 @@ scd_status scd_batch_tune(scd_batch_plan* p, const void* x_arena, const float* w
     scd_status s = try_one(1, p->item_bytes, p->slot_bytes);
     if (s != SCD_OK) return s;
   }
-  if (p->estimator == 1 && p->precision == SCD_FP32) {          // ... with the fused SSCA kernels
+  if (p->precision == SCD_FP32) {                               // ... with the paired transforms
     scd_status s = try_one(2, p->item_bytes, p->slot_bytes);
     if (s != SCD_OK) return s;
   }

@@ -14,8 +14,8 @@
 // product array ever exists in memory), then the P-point FFT, and the fftshifted bins go
 // straight to out[kh][lh][qh].  X (Np*P*8 bytes, 2 MiB at Np=256, P=1024) stays in L2, so
 // the kernel's DRAM traffic is essentially the 8 Np^2 P output bytes.
+#include "fam2.cuh"
 #include "internal.h"
-#include "tiles.cuh"
 
 namespace scd {
 namespace {
@@ -185,6 +185,14 @@ cudaError_t fam_channelise(const float2* x, int Np, int L, int P, const float* w
 
 cudaError_t fam_pair_fft(const float2* X, const float2* Y, int Np, int P, float2* out, cudaStream_t st, int precision) {
   cudaError_t err;
+  if (precision != SCD_SPLIT_BF16 && fam2_supported(P, X == Y)) {
+    FamArgs A{};
+    A.X = X; A.Y = Y; A.out = out; A.Np = Np; A.nsig = 1;
+    if (!(A.tw = table_pass2(P / 2, &err)) || !(A.wP = table_roots(P, &err))) return err;
+    if ((err = fam2_prepare(P)) != cudaSuccess) return err;
+    count_launches(1);
+    return fam2_pairs(A, P, X == Y, false, st);
+  }
   const float2* tw = table_pass(P, &err);
   if (!tw) return err;
   count_launches(1);
@@ -195,6 +203,10 @@ cudaError_t fam_pair_fft(const float2* X, const float2* Y, int Np, int P, float2
     return dispatch_k2<true>(P, X, Y, Np, out, tw, bm, ew, st);
   }
   return dispatch_k2<false>(P, X, Y, Np, out, tw, nullptr, nullptr, st);
+}
+
+bool fam_pair_tables(int P, cudaError_t* err) {
+  return !fam2_supported(P, true) || (table_pass2(P / 2, err) && table_roots(P, err));
 }
 
 cudaError_t fam_channelise_with(const float2* x, int Np, int L, int P, const float* window, float2* X,

@@ -69,26 +69,29 @@ __host__ __device__ __forceinline__ C2 c2_from(float4 q) {
 }
 
 // ----------------------------------------------------------------------------- radix plans
-// As Plan (fft.cuh), with radices of at most 16: a thread holds E = r0 element pairs, 4 E registers.
+// As Plan (fft.cuh) with radices of at most 16: a thread holds E = r0 element pairs, 4 E registers.
 template <int M> struct Plan2;
-template <> struct Plan2<16>   { static constexpr int n = 2; static constexpr int r[3] = {4, 4, 0}; };
-template <> struct Plan2<32>   { static constexpr int n = 2; static constexpr int r[3] = {8, 4, 0}; };
-template <> struct Plan2<64>   { static constexpr int n = 2; static constexpr int r[3] = {8, 8, 0}; };
-template <> struct Plan2<128>  { static constexpr int n = 2; static constexpr int r[3] = {16, 8, 0}; };
-template <> struct Plan2<256>  { static constexpr int n = 2; static constexpr int r[3] = {16, 16, 0}; };
-template <> struct Plan2<512>  { static constexpr int n = 3; static constexpr int r[3] = {16, 8, 4}; };
-template <> struct Plan2<1024> { static constexpr int n = 3; static constexpr int r[3] = {16, 8, 8}; };
+#define SCD_PLAN2(M, N, R0, R1, R2) \
+  template <> struct Plan2<M> { static constexpr int n = N; static constexpr int r[3] = {R0, R1, R2}; };
+SCD_PLAN2(16, 2, 4, 4, 0)
+SCD_PLAN2(32, 2, 8, 4, 0)
+SCD_PLAN2(64, 2, 8, 8, 0)
+SCD_PLAN2(128, 2, 16, 8, 0)
+SCD_PLAN2(256, 2, 16, 16, 0)
+SCD_PLAN2(512, 3, 16, 8, 4)
+SCD_PLAN2(1024, 3, 16, 8, 8)
+#undef SCD_PLAN2
 
 template <int M> struct Plan2Info {
-  static constexpr int n = Plan2<M>::n;
-  static constexpr int r0 = Plan2<M>::r[0], r1 = Plan2<M>::r[1], r2 = Plan2<M>::r[2];
+  using PL = Plan2<M>;
+  static constexpr int n = PL::n, r0 = PL::r[0], rl = PL::r[PL::n - 1];
   static constexpr int E = r0, T = M / E;
-  static constexpr int rl = n == 2 ? r1 : r2;              // last radix
-  static constexpr int p(int s) { return s == 0 ? 1 : (s == 1 ? r0 : r0 * r1); }
-  static constexpr int R(int s) { return s == 0 ? r0 : (s == 1 ? r1 : r2); }
-  static constexpr int off(int s) { return s <= 1 ? 0 : r0 * r1; }
-  static constexpr int tw_len() { return n == 2 ? r0 * r1 : r0 * r1 + r0 * r1 * r2; }
-  // t-fast exchange position: one pad element after every r0, so that the 8 threads of a
+  static constexpr int R(int s) { return PL::r[s]; }
+  static constexpr int p(int s) { return s == 0 ? 1 : p(s - 1) * PL::r[s - 1]; }       // before pass s
+  // the pass table: entry (r, k) of pass s >= 1 at off(s) + r p(s) + k, W_{p R}^{k r}
+  static constexpr int off(int s) { return s <= 1 ? 0 : off(s - 1) + p(s - 1) * PL::r[s - 1]; }
+  static constexpr int tw_len() { return off(n); }
+  // consecutive exchange position: one pad element after every r0, so that the 8 threads of a
   // quarter-warp (the unit of a 16-byte shared-memory access) storing their pass-0 outputs at
   // stride r0 hit 8 different 16-byte banks
   static constexpr int lr0 = r0 >= 16 ? 4 : (r0 >= 8 ? 3 : 2);
@@ -217,6 +220,24 @@ struct PairFft {
 #pragma unroll
     for (int b = 0; b < B; ++b) dft2<R>(v + b * R);
   }
+  // passes S .. n - 2: inputs from and outputs to the exchange area
+  template <int S>
+  __device__ __forceinline__ static void middle(float4* sm, const float2* tw, int c, int t, C2* v) {
+    if constexpr (S < PI::n - 1) {
+      sync<false>();
+      load<S>(sm, tw, c, t, v);
+      dfts<S>(v);
+      sync<false>();                                       // every read of the pass precedes its writes
+      constexpr int R = PI::R(S), p = PI::p(S);
+#pragma unroll
+      for (int b = 0; b < E / R; ++b) {
+        const int i = t + b * T, k = i & (p - 1);
+#pragma unroll
+        for (int j = 0; j < R; ++j) sm[at(c, (i - k) * R + k + p * j)] = c2_f4(v[b * R + j]);
+      }
+      middle<S + 1>(sm, tw, c, t, v);
+    }
+  }
   // free(): called when this thread has read the last of the exchange area
   template <class Free, class Dst>
   __device__ __forceinline__ static void run(float4* sm, const float2* tw, C2* v, Free&& free, Dst& dst) {
@@ -225,19 +246,7 @@ struct PairFft {
     dft2<PI::r0>(v);
 #pragma unroll
     for (int j = 0; j < PI::r0; ++j) sm[at(c, t * PI::r0 + j)] = c2_f4(v[j]);
-    if constexpr (PI::n == 3) {
-      sync<false>();
-      load<1>(sm, tw, c, t, v);
-      dfts<1>(v);
-      sync<false>();                                       // every read of pass 1 precedes its writes
-      constexpr int R = PI::r1, p = PI::r0;
-#pragma unroll
-      for (int b = 0; b < E / R; ++b) {
-        const int i = t + b * T, k = i & (p - 1);
-#pragma unroll
-        for (int j = 0; j < R; ++j) sm[at(c, (i - k) * R + k + p * j)] = c2_f4(v[b * R + j]);
-      }
-    }
+    middle<1>(sm, tw, c, t, v);
     sync<true>();
     load<L>(sm, tw, co, to, v);
     free();

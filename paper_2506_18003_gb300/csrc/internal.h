@@ -45,6 +45,7 @@ cudaError_t fam_channelise(const float2* x, int Np, int L, int P, const float* w
 // out[kh][lh][qh] = sum_p X[kh][p] conj(Y[lh][p]) W_P^{(q p) mod P}   (Y = X: auto estimate)
 cudaError_t fam_pair_fft(const float2* X, const float2* Y, int Np, int P, float2* out, cudaStream_t st,
                          int precision);
+bool fam_pair_tables(int P, cudaError_t* err);             // builds the tables fam_pair_fft's FP32 form uses
 // The same two kernels with caller-provided tables (pass twiddles of size Np and of size P)
 // instead of the cached ones.
 cudaError_t fam_channelise_with(const float2* x, int Np, int L, int P, const float* window, float2* X,

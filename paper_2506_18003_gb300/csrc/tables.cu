@@ -49,6 +49,12 @@ __global__ void k_pass(float2* out, int M, int r0, int r1, int r2) {
     out[e] = root_fp64(pass_twiddle_exponent(e, M, r0, r1, r2), M);
 }
 
+// One pass of the paired transforms' table: W_{p R}^{k r} at r p + k.
+__global__ void k_pass2(float2* out, int p, int R) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < p * R; e += gridDim.x * blockDim.x)
+    out[e] = root_fp64((int64_t)(e % p) * (e / p), (int64_t)p * R);
+}
+
 // W_N^{c m1'} for c < C, m1' < M1 at [m1'][c] (c m1' < C M1 <= N: no reduction needed)
 __global__ void k_cols(float2* out, int64_t N, int M1, int C) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < M1 * C; e += gridDim.x * blockDim.x) {
@@ -231,18 +237,23 @@ const float2* table_pass(int M, cudaError_t* err) {
   });
 }
 
-// The paired transforms' table (Plan2's radices, same layout).
+// The paired transforms' table (the radices of Plan2<M>, same layout).
 const float2* table_pass2(int M, cudaError_t* err) {
-  PassRadices r{0, 0, 0};
-#define SCD_PR(MM) case MM: r = {Plan2<MM>::r[0], Plan2<MM>::r[1], Plan2<MM>::r[2]}; break;
+  const int* r = nullptr;
+  int n = 0, len = 0;
+#define SCD_PR(MM) case MM: r = Plan2<MM>::r; n = Plan2<MM>::n; len = Plan2Info<MM>::tw_len(); break;
   switch (M) {
     SCD_PR(16) SCD_PR(32) SCD_PR(64) SCD_PR(128) SCD_PR(256) SCD_PR(512) SCD_PR(1024)
     default: *err = cudaErrorInvalidValue; return nullptr;
   }
 #undef SCD_PR
-  const int len = pass_table_len(r.r0, r.r1, r.r2);
   return (const float2*)get_or_build(11, M, 0, 0, sizeof(float2) * (size_t)len, err, [&](void* p, cudaStream_t st) {
-    k_pass<<<grid_for(len), 256, 0, st>>>((float2*)p, M, r.r0, r.r1, r.r2);
+    int at = 0, done = r[0];
+    for (int s = 1; s < n; ++s) {                              // pass s: W_{p R}^{k r} at at + r p + k
+      k_pass2<<<grid_for(done * r[s]), 256, 0, st>>>((float2*)p + at, done, r[s]);
+      at += done * r[s];
+      done *= r[s];
+    }
   });
 }
 
