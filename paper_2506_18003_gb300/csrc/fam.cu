@@ -29,6 +29,10 @@ k_fam_channelise(const float2* __restrict__ x, int L, int P, const float* __rest
   using S = TileShape<NP>;
   using FS = FftSmem<NP, S::C, S::NT, TC>;
   unsigned char* base = reinterpret_cast<unsigned char*>(sm);
+  if constexpr (!TC) {
+    let_next_start();
+    wait_for_previous();
+  }
   TcCtx ctx{};
   if constexpr (TC) ctx = tc_begin<FS::tmem_cols>(base + FS::region0 + FS::bbytes, base + FS::region0, bmats, FS::bbytes, err);
   fam_channelise_tile<NP, TC>(sm, ctx, x, L, P, a, tw, X, blockIdx.x * S::C, conj_out != 0);
@@ -45,6 +49,10 @@ __device__ __forceinline__ void fam_pairs_cta(const float2* __restrict__ X, cons
   using S = TileShape<PP>;
   using FS = FftSmem<PP, S::C, S::NT, TC>;
   unsigned char* base = reinterpret_cast<unsigned char*>(sm);
+  if constexpr (!TC) {
+    let_next_start();
+    wait_for_previous();
+  }
   TcCtx ctx{};
   if constexpr (TC) ctx = tc_begin<FS::tmem_cols>(base + FS::region0 + FS::bbytes, base + FS::region0, bmats, FS::bbytes, err);
   fam_pairs_tile<PP, TC, false, SYM>(sm, ctx, X, Y, Np, out, tw, (int64_t)blockIdx.x * S::C);
@@ -79,7 +87,9 @@ cudaError_t launch_k1(const float2* x, int L, int P, const float* window, const 
   constexpr int sm = FftSmem<NPV, S::C, S::NT, TC>::total;
   cudaError_t e = set_smem(k_fam_channelise<NPV, TC>, sm);
   if (e != cudaSuccess) return e;
-  k_fam_channelise<NPV, TC><<<(P + S::C - 1) / S::C, S::NT, sm, st>>>(x, L, P, window, tw, X, bm, err, conj_out);
+  const unsigned grid = (unsigned)((P + S::C - 1) / S::C);
+  if constexpr (!TC) return launch_dependent(true, k_fam_channelise<NPV, TC>, grid, S::NT, sm, st, x, L, P, window, tw, X, bm, err, conj_out);
+  k_fam_channelise<NPV, TC><<<grid, S::NT, sm, st>>>(x, L, P, window, tw, X, bm, err, conj_out);
   return cudaGetLastError();
 }
 
@@ -110,7 +120,9 @@ cudaError_t launch_k2_t(const float2* X, const float2* Y, int Np, float2* out, c
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
   const int64_t npairs = fam_pair_count<PV>(Np, SYM);
-  kernel<<<(unsigned)((npairs + S::C - 1) / S::C), S::NT, sm, st>>>(X, Y, Np, out, tw, bm, err);
+  const unsigned grid = (unsigned)((npairs + S::C - 1) / S::C);
+  if constexpr (!TC) return launch_dependent(true, kernel, grid, S::NT, sm, st, X, Y, Np, out, tw, bm, err);
+  kernel<<<grid, S::NT, sm, st>>>(X, Y, Np, out, tw, bm, err);
   return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
 // FAM pair transforms of fam2.cuh, for one signal or for the signals of one size of a batch plan.
 #include "fam2.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace scd {
 namespace {
@@ -11,33 +12,25 @@ __global__ void __launch_bounds__(FamPair<PP>::NT, FamPair<PP>::minb) k_fam_pair
   fam_pairs2_cta<PP, SYM, PROF>(fam_sm, A);
 }
 
-template <class K>
-cudaError_t set_smem(K kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
 template <int PP>
 cudaError_t prepare_t() {
-  cudaError_t e = set_smem(k_fam_pairs2<PP, true, false>, FamPair<PP>::smem);
-  if (e == cudaSuccess) e = set_smem(k_fam_pairs2<PP, true, true>, FamPair<PP>::smem);
-  if (e == cudaSuccess) e = set_smem(k_fam_pairs2<PP, false, false>, FamPair<PP>::smem);
+  cudaError_t e = allow_smem<k_fam_pairs2<PP, true, false>>(FamPair<PP>::smem);
+  if (e == cudaSuccess) e = allow_smem<k_fam_pairs2<PP, true, true>>(FamPair<PP>::smem);
+  if (e == cudaSuccess) e = allow_smem<k_fam_pairs2<PP, false, false>>(FamPair<PP>::smem);
   return e;
 }
 
 template <int PP>
 cudaError_t launch_t(const FamArgs& A, bool sym, bool prof, cudaStream_t st) {
   using K = FamPair<PP>;
-  int dev = 0, sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int sms = sm_count(&e);
+  if (!sms) return e;
   const int64_t tiles = (fam_pair_count<0>(A.Np, sym) + K::C - 1) / K::C * A.nsig;
   if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
   const unsigned grid = (unsigned)(tiles < (int64_t)K::minb * sms ? tiles : (int64_t)K::minb * sms);
-  if (prof) k_fam_pairs2<PP, true, true><<<grid, K::NT, K::smem, st>>>(A);
-  else if (sym) k_fam_pairs2<PP, true, false><<<grid, K::NT, K::smem, st>>>(A);
-  else k_fam_pairs2<PP, false, false><<<grid, K::NT, K::smem, st>>>(A);
-  return cudaGetLastError();
+  return launch_dependent(true, prof ? k_fam_pairs2<PP, true, true> : (sym ? k_fam_pairs2<PP, true, false> : k_fam_pairs2<PP, false, false>),
+                          grid, K::NT, K::smem, st, A);
 }
 
 }  // namespace

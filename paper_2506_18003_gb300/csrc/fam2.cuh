@@ -16,6 +16,7 @@
 // shared-memory pipe (77% of its cycles) with 16 warps per SM.
 #pragma once
 #include "fft2.cuh"
+#include "pdl.cuh"
 #include "tiles.cuh"
 
 namespace scd {
@@ -70,8 +71,10 @@ __device__ __forceinline__ void fam_pairs2_cta(unsigned char* sm, const FamArgs&
 #pragma unroll
   for (int b = 0; b < B; ++b) wb[b] = __ldg(A.wP + t + b * T);
   const int npairs = (int)fam_pair_count<0>(Np, SYM), per = (npairs + C - 1) / C, tiles = per * A.nsig;
+  wait_for_previous();
   __syncthreads();
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (tile + (int)gridDim.x >= tiles) let_next_start();   // this CTA's last tile
     const int s = tile / per, pair = (tile - s * per) * C + c;
     const FamSig g = A.sig ? A.sig[s] : FamSig{0, 0};
     const bool valid = pair < npairs;

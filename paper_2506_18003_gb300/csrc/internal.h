@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "../../include/scd.h"
@@ -157,6 +158,27 @@ struct NvtxRange {
   explicit NvtxRange(const char* name);
   ~NvtxRange();
 };
+
+// ---------------------------------------------------------------- per-device launch state
+// Changes with every scd_release_cache(), after which everything kept per device is set up anew.
+unsigned cache_generation();
+constexpr int kKeptDevices = 32;
+// Streaming multiprocessors of the current device, asked for once.
+int sm_count(cudaError_t* err);
+// Dynamic shared memory limit of kernel K on the current device, set once (the call costs as much host
+// time as a quarter of a launch).
+template <auto K>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<unsigned> done[kKeptDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned now = cache_generation() + 1u;
+  if (dev < kKeptDevices && done[dev].load(std::memory_order_acquire) == now) return cudaSuccess;
+  e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev < kKeptDevices) done[dev].store(now, std::memory_order_release);
+  return e;
+}
 
 // ---------------------------------------------------------------- launch accounting
 void count_launches(int n);

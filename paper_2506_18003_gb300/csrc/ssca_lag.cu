@@ -1,6 +1,7 @@
 // SSCA auto estimates in the lag domain: the kernels of ssca_lag.cuh's three passes, for one signal or
 // for the signals of one size of a batch plan.
 #include "internal.h"
+#include "pdl.cuh"
 #include "ssca_lag.cuh"
 
 namespace scd {
@@ -23,19 +24,13 @@ k_lag_chan(const LagArgs A, const __grid_constant__ CUtensorMap tp, const __grid
   lag_chan_cta<NP, NTHR, PROF>(lag_sm, A, &tp, &tn);
 }
 
-template <class K>
-cudaError_t set_smem(K kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
 // persistent CTAs of a launch over `tiles` tiles: per_sm of nt threads on every SM, of a large output at
 // most 512 threads
 cudaError_t grid_of(const LagArgs& A, int64_t tiles, int per_sm, int nt, unsigned* grid) {
   if (lag_large(A.N, A.Np, A.nsig) && per_sm * nt > 512) per_sm = 512 / nt;
-  int dev = 0, sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int sms = sm_count(&e);
+  if (!sms) return e;
   *grid = (unsigned)(tiles < (int64_t)per_sm * sms ? tiles : (int64_t)per_sm * sms);
   return cudaSuccess;
 }
@@ -46,8 +41,7 @@ template <int M1>
 cudaError_t launch_cols(const LagArgs& A, cudaStream_t st) {
   const int64_t tiles = (int64_t)lag_cols_tiles(A.np, M1, A.M2) * A.nsig;
   if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
-  k_lag_cols<M1><<<(unsigned)tiles, LagCols<M1>::NT, LagCols<M1>::smem, st>>>(A);
-  return cudaGetLastError();
+  return launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_cols<M1>, (unsigned)tiles, LagCols<M1>::NT, LagCols<M1>::smem, st, A);
 }
 
 template <int M2>
@@ -58,8 +52,7 @@ cudaError_t launch_rows(const LagArgs& A, cudaStream_t st) {
   unsigned grid;
   cudaError_t e = grid_of(A, tiles, K::minb, K::NT, &grid);
   if (e != cudaSuccess) return e;
-  k_lag_rows<M2><<<grid, K::NT, K::smem, st>>>(A);
-  return cudaGetLastError();
+  return launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_rows<M2>, grid, K::NT, K::smem, st, A);
 }
 
 template <int NP, int NTHR>
@@ -76,9 +69,8 @@ cudaError_t launch_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st
   const cuuint32_t bp[3] = {K::pos_row, NP / 2, 1}, bn[3] = {K::neg_row, NP / 2, 1};
   if ((e = encode_map_c64(&tp, A.R + r0, 3, dims, strides, bp)) != cudaSuccess) return e;
   if ((e = encode_map_c64(&tn, A.R + r0, 3, dims, strides, bn)) != cudaSuccess) return e;
-  if (prof) k_lag_chan<NP, NTHR, true><<<grid, K::NT, K::smem, st>>>(A, tp, tn);
-  else k_lag_chan<NP, NTHR, false><<<grid, K::NT, K::smem, st>>>(A, tp, tn);
-  return cudaGetLastError();
+  return prof ? launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_chan<NP, NTHR, true>, grid, K::NT, K::smem, st, A, tp, tn)
+              : launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_chan<NP, NTHR, false>, grid, K::NT, K::smem, st, A, tp, tn);
 }
 
 }  // namespace
@@ -86,14 +78,14 @@ cudaError_t launch_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st
 cudaError_t lag_prepare(int M1, int M2, int Np) {
   cudaError_t e = cudaErrorInvalidValue;
   switch (M1) {
-#define SCD_X(M) case M: e = set_smem(k_lag_cols<M>, LagCols<M>::smem); break;
+#define SCD_X(M) case M: e = allow_smem<k_lag_cols<M>>(LagCols<M>::smem); break;
     SCD_LAG_STRIP(SCD_X)
 #undef SCD_X
   }
   if (e != cudaSuccess) return e;
   e = cudaErrorInvalidValue;
   switch (M2) {
-#define SCD_X(M) case M: e = set_smem(k_lag_rows<M>, LagRows<M>::smem); break;
+#define SCD_X(M) case M: e = allow_smem<k_lag_rows<M>>(LagRows<M>::smem); break;
     SCD_LAG_STRIP(SCD_X)
 #undef SCD_X
   }
@@ -101,8 +93,8 @@ cudaError_t lag_prepare(int M1, int M2, int Np) {
   e = cudaErrorInvalidValue;
   switch (Np) {
 #define SCD_X(M, T)                                                                                \
-  if (e == cudaSuccess) e = set_smem(k_lag_chan<M, T, false>, LagChan<M, T>::smem);               \
-  if (e == cudaSuccess) e = set_smem(k_lag_chan<M, T, true>, LagChan<M, T>::smem);
+  if (e == cudaSuccess) e = allow_smem<k_lag_chan<M, T, false>>(LagChan<M, T>::smem);               \
+  if (e == cudaSuccess) e = allow_smem<k_lag_chan<M, T, true>>(LagChan<M, T>::smem);
     case 16: e = cudaSuccess; SCD_X(16, 128) break;
     case 32: e = cudaSuccess; SCD_X(32, 128) break;
     case 64: e = cudaSuccess; SCD_X(64, 128) break;

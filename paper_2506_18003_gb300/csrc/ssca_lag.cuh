@@ -31,6 +31,7 @@
 // and S out: 3 x 8 Np N bytes, of which only S must reach HBM while the intermediate fits L2.
 #pragma once
 #include "fft2.cuh"
+#include "pdl.cuh"
 #include "tma.cuh"
 
 namespace scd {
@@ -169,6 +170,7 @@ __device__ __forceinline__ void lag_cols_tile(unsigned char* sm, const LagArgs& 
   float2 rot[B];
 #pragma unroll
   for (int b = 0; b < B; ++b) rot[b] = __ldg(A.wN + m2 * (t + b * T));
+  wait_for_previous();
   C2 v[E];
   const float2* xp = A.x + g.x + (t * M2 + m2);
 #pragma unroll
@@ -190,7 +192,7 @@ __device__ __forceinline__ void lag_cols_tile(unsigned char* sm, const LagArgs& 
   auto dst = [&](int b, int j, int f, const C2& val) {
     *at_bytes(yo, 16u * (uint32_t)(f * M2 + m2)) = c2_f4(cmul(val, cmul(rot[b], stage[j * C + c])));
   };
-  K::F::run(reinterpret_cast<float4*>(sm), tws, v, [] {}, dst);
+  K::F::run(reinterpret_cast<float4*>(sm), tws, v, [] { let_next_start(); }, dst);
 }
 
 // Row pass: persistent over the tiles of C rows (pair, q1).
@@ -211,6 +213,7 @@ __device__ __forceinline__ void lag_rows_cta(unsigned char* sm, const LagArgs& A
     fence_mbar_init();
   }
   for (int e = threadIdx.x; e < K::PI::tw_len(); e += K::NT) tws[e] = __ldg(A.tw + e);
+  wait_for_previous();
   __syncthreads();
   if (threadIdx.x == 0 && (int)blockIdx.x < tiles) issue(blockIdx.x);
   uint32_t phase = 0u;
@@ -218,6 +221,7 @@ __device__ __forceinline__ void lag_rows_cta(unsigned char* sm, const LagArgs& A
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const bool got = umma::mbar_wait_bounded(mbar, phase, kMbarPollLimit);
     if (__syncthreads_or(!got)) { ok = false; break; }      // one decision for the whole CTA
+    if (tile + (int)gridDim.x >= tiles) let_next_start();   // this CTA's last tile
     phase ^= 1u;
     C2 v[E];
     {
@@ -299,6 +303,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
     const float2 s0 = __ldg(A.wN + ((-d * l) & (N - 1))), s1 = __ldg(A.wN + ((-(d + 1) * l) & (N - 1)));
     step[e] = make_float4(s0.x, s1.x, s0.y, s1.y);
   }
+  wait_for_previous();
   __syncthreads();
   if (threadIdx.x == 0 && (int)blockIdx.x < tiles) issue(blockIdx.x);
   float2 next = lag <= H && (int)blockIdx.x < tiles ? root(blockIdx.x) : make_float2(0.f, 0.f);
@@ -310,6 +315,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
     if (lag <= H) turn[lag - 1] = cscale(next, alag);
     const bool got = umma::mbar_wait_bounded(mbar, phase, kMbarPollLimit);
     if (__syncthreads_or(!got)) { ok = false; break; }      // one decision for the whole CTA
+    if (tile + (int)gridDim.x >= tiles) let_next_start();   // this CTA's last tile
     phase ^= 1u;
     C2 v[E];
     {                                                       // lags m = t + i S0 >= 0

@@ -9,6 +9,7 @@
 // order).  Each entry is computed once with FP64
 // sincospi(2 j / M) (argument exact: M is a power of two) and rounded to float32, so no
 // phase ever loses accuracy to an FP32 angle, even at M = 2^20.
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -177,6 +178,7 @@ struct Key {
 
 std::mutex g_mu;
 std::map<Key, void*> g_tables;
+std::atomic<unsigned> g_generation{0};
 
 struct PassRadices { int r0, r1, r2; };
 PassRadices pass_radices(int M) {
@@ -350,8 +352,25 @@ unsigned* device_error_word(cudaError_t* err) {
   });
 }
 
+unsigned cache_generation() { return g_generation.load(std::memory_order_acquire); }
+
+int sm_count(cudaError_t* err) {
+  static std::atomic<uint64_t> kept[kKeptDevices] = {};         // generation + 1 above the count
+  int dev = 0, n = 0;
+  if ((*err = cudaGetDevice(&dev)) != cudaSuccess) return 0;
+  const uint64_t now = (uint64_t)cache_generation() + 1u;
+  if (dev < kKeptDevices) {
+    const uint64_t k = kept[dev].load(std::memory_order_acquire);
+    if (k >> 32 == now) return (int)(k & 0xFFFFFFFFu);
+  }
+  if ((*err = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return 0;
+  if (dev < kKeptDevices) kept[dev].store(now << 32 | (uint64_t)n, std::memory_order_release);
+  return n;
+}
+
 void release_tables() {
   std::lock_guard<std::mutex> lock(g_mu);
+  g_generation.fetch_add(1, std::memory_order_acq_rel);
   int cur = 0;
   cudaGetDevice(&cur);
   for (auto& kv : g_tables) {
