@@ -353,7 +353,8 @@ scd_status scd_prepare(int32_t estimator, int64_t N, int32_t Np, int32_t P) {
       return scd::table_pass(P, &e) && scd::fam_pair_tables(P, &e) ? SCD_OK : cuda_fail(e);
     }
     const int64_t M = scd::bluestein_len_host(P);
-    if (!scd::table_pass((int)M, &e) || !scd::table_chirp(P, &e) || !scd::table_bluestein(P, M, &e))
+    if (!scd::table_pass((int)M, &e) || (M >= 64 && M <= 4096 && !scd::table_pass_sym((int)M, &e)) ||
+        !scd::table_chirp(P, &e) || !scd::table_bluestein(P, M, &e))
       return cuda_fail(e);
     return SCD_OK;
   }

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "bluestein.cuh"
+#include "bluestein2.cuh"
 #include "internal.h"
 
 namespace scd {
@@ -71,15 +72,6 @@ k_fam_pairs_any(const float2* __restrict__ X, const float2* __restrict__ Y, int 
   fam_pairs_any_cta<MM, TC>(X, Y, Np, P, out, tw, chirp, bh, bmats, err);
 }
 
-// The same kernel held to 128 registers per thread, so that two 256-thread CTAs share an SM.
-template <int MM, bool TC>
-__global__ void __launch_bounds__(TileShape<MM>::NT, 2)
-k_fam_pairs_any_2cta(const float2* __restrict__ X, const float2* __restrict__ Y, int Np, int P,
-                     float2* __restrict__ out, const float2* __restrict__ tw, const float2* __restrict__ chirp,
-                     const float2* __restrict__ bh, const unsigned char* __restrict__ bmats, unsigned* err) {
-  fam_pairs_any_cta<MM, TC>(X, Y, Np, P, out, tw, chirp, bh, bmats, err);
-}
-
 template <class K>
 cudaError_t launch_fam_any_k(K kernel, int smem, int NT, int C, const float2* X, const float2* Y, int Np, int P,
                              float2* out, const float2* tw, const float2* chirp, const float2* bh, TcArgs t,
@@ -91,18 +83,40 @@ cudaError_t launch_fam_any_k(K kernel, int smem, int NT, int C, const float2* X,
   return cudaGetLastError();
 }
 
-// The FP32 form from MM = 2048 runs two CTAs per SM (Np = 256, P = 1000: 0.86 -> 0.64 ms;
-// Np = 64, P = 4000: 0.24 -> 0.21 ms); below MM = 2048 the register cap spills, and the
-// tensor-core form lost time under it.
 template <int MM, bool TC>
 cudaError_t launch_fam_any(const float2* X, const float2* Y, int Np, int P, float2* out, const float2* tw,
                            const float2* chirp, const float2* bh, TcArgs t, cudaStream_t st) {
   using S = TileShape<MM>;
   constexpr int sm = ResidentSmem<MM, TC>::total;
-  if constexpr (!TC && MM >= 2048 && S::NT <= 256)
-    return launch_fam_any_k(k_fam_pairs_any_2cta<MM, TC>, sm, S::NT, S::C, X, Y, Np, P, out, tw, chirp, bh, t, st);
-  else
-    return launch_fam_any_k(k_fam_pairs_any<MM, TC>, sm, S::NT, S::C, X, Y, Np, P, out, tw, chirp, bh, t, st);
+  return launch_fam_any_k(k_fam_pairs_any<MM, TC>, sm, S::NT, S::C, X, Y, Np, P, out, tw, chirp, bh, t, st);
+}
+
+// Two pairs at a time on the packed lanes (bluestein2.cuh): the FP32 form, cyclic lengths 64 .. 4096.
+template <int M, bool SYM>
+__global__ void __launch_bounds__(FamAny2<M>::NT, FamAny2<M>::minb)
+k_fam_any2(const float2* __restrict__ X, const float2* __restrict__ Y, int Np, int P, float2* __restrict__ out,
+           const float2* __restrict__ tw, const float2* __restrict__ chirp, const float2* __restrict__ bh) {
+  extern __shared__ __align__(128) unsigned char any2_sm[];
+  fam_any2_cta<M, SYM>(any2_sm, X, Y, Np, P, out, tw, chirp, bh);
+}
+
+template <int M>
+cudaError_t launch_fam_any2(const float2* X, const float2* Y, int Np, int P, float2* out, const float2* chirp,
+                            const float2* bh, cudaStream_t st) {
+  using K = FamAny2<M>;
+  cudaError_t e;
+  const float2* tw = table_pass_sym(M, &e);
+  if (!tw) return e;
+  const int sms = sm_count(&e);
+  if (!sms) return e;
+  if ((e = allow_smem<k_fam_any2<M, true>>(K::smem)) != cudaSuccess ||
+      (e = allow_smem<k_fam_any2<M, false>>(K::smem)) != cudaSuccess)
+    return e;
+  const bool sym = X == Y;                                     // the auto estimate: pairs kh <= lh
+  const int64_t tiles = (fam_pair_count<0>(Np, sym) / 2 + K::C - 1) / K::C;
+  const unsigned grid = (unsigned)(tiles < (int64_t)K::minb * sms ? tiles : (int64_t)K::minb * sms);
+  return launch_dependent(true, sym ? k_fam_any2<M, true> : k_fam_any2<M, false>, grid, K::NT, K::smem, st, X, Y, Np, P,
+                          out, tw, chirp, bh);
 }
 
 // ---------------------------------------------------------------- SSCA
@@ -280,23 +294,20 @@ cudaError_t fam_pair_fft_any(const float2* X, const float2* Y, int Np, int P, fl
   TcArgs t;
   if ((err = tc_args(tc, (int)MM, &t)) != cudaSuccess) return err;
   count_launches(1);
-#define SCD_FA(MV) return tc ? launch_fam_any<MV, true>(X, Y, Np, P, out, tw, chirp, bh, t, st) \
-                             : launch_fam_any<MV, false>(X, Y, Np, P, out, tw, chirp, bh, t, st)
-  switch (MM) {
-    case 8: SCD_FA(8);
-    case 16: SCD_FA(16);
-    case 32: SCD_FA(32);
-    case 64: SCD_FA(64);
-    case 128: SCD_FA(128);
-    case 256: SCD_FA(256);
-    case 512: SCD_FA(512);
-    case 1024: SCD_FA(1024);
-    case 2048: SCD_FA(2048);
-    case 4096: SCD_FA(4096);
-    case 8192: SCD_FA(8192);
-    case 16384: SCD_FA(16384);
+#define SCD_FA(MV, TC) case MV: return launch_fam_any<MV, TC>(X, Y, Np, P, out, tw, chirp, bh, t, st);
+#define SCD_F2(MV) case MV: return launch_fam_any2<MV>(X, Y, Np, P, out, chirp, bh, st);
+  if (tc) switch (MM) {
+    SCD_FA(8, true) SCD_FA(16, true) SCD_FA(32, true) SCD_FA(64, true) SCD_FA(128, true) SCD_FA(256, true)
+    SCD_FA(512, true) SCD_FA(1024, true) SCD_FA(2048, true) SCD_FA(4096, true) SCD_FA(8192, true) SCD_FA(16384, true)
     default: return cudaErrorInvalidValue;
   }
+  switch (MM) {
+    SCD_FA(8, false) SCD_FA(16, false) SCD_FA(32, false)
+    SCD_F2(64) SCD_F2(128) SCD_F2(256) SCD_F2(512) SCD_F2(1024) SCD_F2(2048) SCD_F2(4096)
+    SCD_FA(8192, false) SCD_FA(16384, false)
+    default: return cudaErrorInvalidValue;
+  }
+#undef SCD_F2
 #undef SCD_FA
 }
 

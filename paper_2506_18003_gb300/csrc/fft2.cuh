@@ -81,9 +81,22 @@ SCD_PLAN2(256, 2, 16, 16, 0)
 SCD_PLAN2(512, 3, 16, 8, 4)
 SCD_PLAN2(1024, 3, 16, 8, 8)
 #undef SCD_PLAN2
+// Plans whose last radix is the first: the bins that a thread gets from the last pass are the inputs that
+// the first pass of another transform of the size takes from it (any-length transforms, bluestein2.cuh).
+template <int M> struct PlanSym;
+#define SCD_PLAN_SYM(M, N, R0, R1, R2) \
+  template <> struct PlanSym<M> { static constexpr int n = N; static constexpr int r[3] = {R0, R1, R2}; };
+SCD_PLAN_SYM(64, 2, 8, 8, 0)
+SCD_PLAN_SYM(128, 3, 8, 2, 8)
+SCD_PLAN_SYM(256, 2, 16, 16, 0)
+SCD_PLAN_SYM(512, 3, 16, 2, 16)
+SCD_PLAN_SYM(1024, 3, 16, 4, 16)
+SCD_PLAN_SYM(2048, 3, 16, 8, 16)
+SCD_PLAN_SYM(4096, 3, 16, 16, 16)
+#undef SCD_PLAN_SYM
 
-template <int M> struct Plan2Info {
-  using PL = Plan2<M>;
+template <int M, template <int> class PlanT = Plan2> struct Plan2Info {
+  using PL = PlanT<M>;
   static constexpr int n = PL::n, r0 = PL::r[0], rl = PL::r[PL::n - 1];
   static constexpr int E = r0, T = M / E;
   static constexpr int R(int s) { return PL::r[s]; }
@@ -148,6 +161,20 @@ __host__ __device__ __forceinline__ void unscramble2(C2* v) {
     unscramble2<R, I + 1>(v);
   }
 }
+template <int R, int J>
+__host__ __device__ __forceinline__ void spread2(C2* v) {       // the first stage on v[R / 2 ..] = 0
+  if constexpr (J < R / 2) {
+    v[J + R / 2] = twc2<R, J>(v[J]);
+    spread2<R, J + 1>(v);
+  }
+}
+// R-point DFT whose inputs from R / 2 on are zero (v[R / 2 ..] not read).
+template <int R>
+__host__ __device__ __forceinline__ void dft2_half(C2* v) {
+  spread2<R, 0>(v);
+  dif2_all<R, R / 4>(v);
+  unscramble2<R, 0>(v);
+}
 template <int R>
 __host__ __device__ __forceinline__ void dft2(C2* v) {
   dif2_all<R, R / 2>(v);
@@ -168,9 +195,9 @@ enum PairMap { kInterleaved, kConsecutive, kRowsToCols };
 // v holds the pass-0 inputs t + r (M / r0) of this thread's pair; dst(b, j, f, value) receives bin f
 // = i + p j, i = t + b T, p = M / rl, b < E / rl, j < rl of the last pass's thread (c, t) = out_c(),
 // out_t().  Callers that run several batches put a barrier between them.
-template <int M, int C, int MAP>
+template <int M, int C, int MAP, template <int> class PlanT = Plan2>
 struct PairFft {
-  using PI = Plan2Info<M>;
+  using PI = Plan2Info<M, PlanT>;
   static constexpr int E = PI::E, T = PI::T;
   static constexpr int tstride = (M + M / PI::r0) | 1;
   static constexpr int smem_f4 = MAP == kInterleaved ? M * C : tstride * C;
@@ -238,23 +265,30 @@ struct PairFft {
       middle<S + 1>(sm, tw, c, t, v);
     }
   }
-  // free(): called when this thread has read the last of the exchange area
-  template <class Free, class Dst>
-  __device__ __forceinline__ static void run(float4* sm, const float2* tw, C2* v, Free&& free, Dst& dst) {
-    constexpr int L = PI::n - 1, RL = PI::rl;
-    const int c = in_c(), t = in_t(), co = out_c(), to = out_t();
-    dft2<PI::r0>(v);
+  // The transform up to its last pass's results in v[b rl + j]; free(): called when this thread has read
+  // the last of the exchange area.
+  // HALF: the inputs M / 2 .. M - 1 (v[r0 / 2 ..]) are zero and not read.
+  template <bool HALF = false, class Free>
+  __device__ __forceinline__ static void transform(float4* sm, const float2* tw, C2* v, Free&& free) {
+    const int c = in_c(), t = in_t();
+    if constexpr (HALF) dft2_half<PI::r0>(v);
+    else dft2<PI::r0>(v);
 #pragma unroll
     for (int j = 0; j < PI::r0; ++j) sm[at(c, t * PI::r0 + j)] = c2_f4(v[j]);
     middle<1>(sm, tw, c, t, v);
     sync<true>();
-    load<L>(sm, tw, co, to, v);
+    load<PI::n - 1>(sm, tw, out_c(), out_t(), v);
     free();
-    dfts<L>(v);
+    dfts<PI::n - 1>(v);
+  }
+  template <class Free, class Dst>
+  __device__ __forceinline__ static void run(float4* sm, const float2* tw, C2* v, Free&& free, Dst& dst) {
+    constexpr int RL = PI::rl;
+    transform(sm, tw, v, free);
 #pragma unroll
     for (int b = 0; b < E / RL; ++b)
 #pragma unroll
-      for (int j = 0; j < RL; ++j) dst(b, j, to + b * T + (M / RL) * j, v[b * RL + j]);
+      for (int j = 0; j < RL; ++j) dst(b, j, out_t() + b * T + (M / RL) * j, v[b * RL + j]);
   }
 };
 

@@ -239,17 +239,10 @@ const float2* table_pass(int M, cudaError_t* err) {
   });
 }
 
-// The paired transforms' table (the radices of Plan2<M>, same layout).
-const float2* table_pass2(int M, cudaError_t* err) {
-  const int* r = nullptr;
-  int n = 0, len = 0;
-#define SCD_PR(MM) case MM: r = Plan2<MM>::r; n = Plan2<MM>::n; len = Plan2Info<MM>::tw_len(); break;
-  switch (M) {
-    SCD_PR(16) SCD_PR(32) SCD_PR(64) SCD_PR(128) SCD_PR(256) SCD_PR(512) SCD_PR(1024)
-    default: *err = cudaErrorInvalidValue; return nullptr;
-  }
-#undef SCD_PR
-  return (const float2*)get_or_build(11, M, 0, 0, sizeof(float2) * (size_t)len, err, [&](void* p, cudaStream_t st) {
+// The paired transforms' tables (the radices of Plan2<M> or PlanSym<M>, same layout).
+static const float2* pass2_table(int kind, int M, const int* r, int n, int len, cudaError_t* err) {
+  if (!r) { *err = cudaErrorInvalidValue; return nullptr; }
+  return (const float2*)get_or_build(kind, M, 0, 0, sizeof(float2) * (size_t)len, err, [&](void* p, cudaStream_t st) {
     int at = 0, done = r[0];
     for (int s = 1; s < n; ++s) {                              // pass s: W_{p R}^{k r} at at + r p + k
       k_pass2<<<grid_for(done * r[s]), 256, 0, st>>>((float2*)p + at, done, r[s]);
@@ -257,6 +250,24 @@ const float2* table_pass2(int M, cudaError_t* err) {
       done *= r[s];
     }
   });
+}
+
+const float2* table_pass2(int M, cudaError_t* err) {
+  switch (M) {
+#define SCD_PR(MM) case MM: return pass2_table(11, M, Plan2<MM>::r, Plan2<MM>::n, Plan2Info<MM>::tw_len(), err);
+    SCD_PR(16) SCD_PR(32) SCD_PR(64) SCD_PR(128) SCD_PR(256) SCD_PR(512) SCD_PR(1024)
+#undef SCD_PR
+    default: *err = cudaErrorInvalidValue; return nullptr;
+  }
+}
+
+const float2* table_pass_sym(int M, cudaError_t* err) {
+  switch (M) {
+#define SCD_PR(MM) case MM: return pass2_table(12, M, PlanSym<MM>::r, PlanSym<MM>::n, Plan2Info<MM, PlanSym>::tw_len(), err);
+    SCD_PR(64) SCD_PR(128) SCD_PR(256) SCD_PR(512) SCD_PR(1024) SCD_PR(2048) SCD_PR(4096)
+#undef SCD_PR
+    default: *err = cudaErrorInvalidValue; return nullptr;
+  }
 }
 
 const float2* table_cols(int N, int M1, int C, cudaError_t* err) {
