@@ -356,7 +356,7 @@ scd_status scd_prepare(int32_t estimator, int64_t N, int32_t Np, int32_t P) {
     if (!scd::table_pass((int)M, &e) || (M >= 64 && M <= 4096 && !scd::table_pass_sym((int)M, &e)) ||
         !scd::table_chirp(P, &e) || !scd::table_bluestein(P, M, &e))
       return cuda_fail(e);
-    return SCD_OK;
+    return scd::prepare_mix(P, &e) ? SCD_OK : cuda_fail(e);
   }
   if (estimator == 1) {
     if (N < 4096 || N > (1 << 20) || (!scd::is_pow2(N) && N > kMaxAnyN)) return SCD_ERR_UNSUPPORTED;

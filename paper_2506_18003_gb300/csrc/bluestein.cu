@@ -21,6 +21,7 @@
 
 #include "bluestein.cuh"
 #include "bluestein2.cuh"
+#include "mix2.cuh"
 #include "internal.h"
 
 namespace scd {
@@ -282,6 +283,8 @@ AnyLayout any_layout(int64_t N, int Np, void* ws) {
 
 cudaError_t fam_pair_fft_any(const float2* X, const float2* Y, int Np, int P, float2* out, cudaStream_t st,
                              int precision) {
+  MixPlan plan;
+  if (precision != SCD_SPLIT_BF16 && mix_plan(P, &plan)) return fam_mix_pairs(X, Y, Np, plan, out, st);
   const int64_t MM = bluestein_len(P);
   cudaError_t err;
   const float2* tw = table_pass((int)MM, &err);

@@ -36,19 +36,6 @@ struct FamAny2 {
   static constexpr int minb = PI::E >= 16 ? 512 / NT : 1024 / NT;
 };
 
-// (kh, lh) of pair number `pair`: all Np^2, or (SYM) the folded triangle kh <= lh (fam_pairs_tile)
-template <bool SYM>
-__device__ __forceinline__ void fam_pair_of(int pair, int Np, int* kh, int* lh) {
-  if constexpr (SYM) {
-    const int r = pair / (Np + 1), c = pair - r * (Np + 1);
-    if (c < Np - r) { *kh = r; *lh = r + c; }
-    else { *kh = Np - 1 - r; *lh = c - 1; }
-  } else {
-    *kh = pair / Np;
-    *lh = pair - *kh * Np;
-  }
-}
-
 // Persistent over the pairs two by two (their number is even).
 template <int M, bool SYM>
 __device__ __forceinline__ void fam_any2_cta(unsigned char* smem, const float2* __restrict__ X,

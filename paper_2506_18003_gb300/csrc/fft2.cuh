@@ -68,6 +68,18 @@ __host__ __device__ __forceinline__ C2 c2_from(float4 q) {
   return C2{make_float2(q.x, q.y), make_float2(q.z, q.w)};
 }
 
+// One 16-byte load: from plain C++ the compiler makes two 8-byte ones, each of which then walks the
+// 16-byte elements at half the bank bandwidth.
+__device__ __forceinline__ C2 take2(const float4* p) {
+#if defined(__CUDA_ARCH__)
+  unsigned long long re, im;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(re), "=l"(im) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+  return C2{f2_from(re), f2_from(im)};
+#else
+  return c2_from(*p);
+#endif
+}
+
 // ----------------------------------------------------------------------------- radix plans
 // As Plan (fft.cuh) with radices of at most 16: a thread holds E = r0 element pairs, 4 E registers.
 template <int M> struct Plan2;
@@ -215,17 +227,6 @@ struct PairFft {
     team_sync<T, MAP == kInterleaved || (LAST && MAP == kRowsToCols)>();
   }
 
-  // One 16-byte load: from plain C++ the compiler makes two 8-byte ones, each of which then walks the
-  // 16-byte elements at half the bank bandwidth.
-  __device__ __forceinline__ static C2 take(const float4* p) {
-#if defined(__CUDA_ARCH__)
-    unsigned long long re, im;
-    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(re), "=l"(im) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
-    return C2{f2_from(re), f2_from(im)};
-#else
-    return c2_from(*p);
-#endif
-  }
   // Twiddled inputs of pass S (tw: the pass table, in shared memory) and its radix transforms.
   template <int S>
   __device__ __forceinline__ static void load(const float4* sm, const float2* tw, int c, int t, C2* v) {
@@ -235,7 +236,7 @@ struct PairFft {
       const int i = t + b * T, k = i & (p - 1);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        C2 x = take(sm + at(c, i + r * (M / R)));
+        C2 x = take2(sm + at(c, i + r * (M / R)));
         if (r > 0) x = cmul(x, tw[PI::off(S) + r * p + k]);
         v[b * R + r] = x;
       }

@@ -20,6 +20,9 @@ const float2* table_roots(int M, cudaError_t* err);        // W_M^j, j in [0, M)
 const float2* table_pass(int M, cudaError_t* err);         // Stockham pass twiddles of a size-M FFT
 const float2* table_pass2(int M, cudaError_t* err);        // ... of a paired size-M FFT (fft2.cuh)
 const float2* table_pass_sym(int M, cudaError_t* err);     // ... with the plan PlanSym<M>
+struct MixPlan;
+const float2* table_mix(const MixPlan& plan, cudaError_t* err);   // mixed-radix twiddles (mix2.cuh)
+bool prepare_mix(int P, cudaError_t* err);                 // ... built if P has such a plan
 const float2* table_cols(int N, int M1, int C, cudaError_t* err);  // W_N^{c m1'}, [m1'][c], c < C
 const float* table_hamming(int Np, cudaError_t* err);      // default window, float32
 // Bluestein tables of a length-N DFT carried by size-M transforms (M a power of two >= 2N - 1):

@@ -227,7 +227,7 @@ __device__ __forceinline__ void lag_rows_cta(unsigned char* sm, const LagArgs& A
     {
       const float4* row = reinterpret_cast<const float4*>(sm) + K::F::in_c() * M2 + K::F::in_t();
 #pragma unroll
-      for (int r = 0; r < E; ++r) v[r] = K::F::take(row + r * (M2 / E));
+      for (int r = 0; r < E; ++r) v[r] = take2(row + r * (M2 / E));
     }
     __syncthreads();                                        // the landing area becomes the exchange area
     const LagSig g = lag_sig(A, tile / sig_tiles);
@@ -322,7 +322,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
       const float4* pos = reinterpret_cast<const float4*>(sm) + t * C + c;
 #pragma unroll
       for (int i = 0; i < E / 2; ++i) {
-        const C2 r = K::F::take(pos + i * S0 * C);          // (re, im) of f0, of f0 + 1
+        const C2 r = take2(pos + i * S0 * C);          // (re, im) of f0, of f0 + 1
         const float w = win[t + i * S0];
         v[i] = c2_pack(cscale(r.re, w), cscale(r.im, w));
       }
@@ -336,7 +336,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
         float2 r0 = neg[-i * S0 * K::neg_row];
         const float2 r1 = neg[-i * S0 * K::neg_row - 1];
         if (wrap) r0 = __ldg(r0p - i * S0 * N);
-        const C2 f = cmul(i ? cmul(u, K::F::take(step + i * C + c)) : u, turn[mh - 1 - i * S0]);
+        const C2 f = cmul(i ? cmul(u, take2(step + i * C + c)) : u, turn[mh - 1 - i * S0]);
         v[E / 2 + i] = c2_pack(cmulc(c2_lane0(f), r0), cmulc(c2_lane1(f), r1));
       }
     }

@@ -20,6 +20,7 @@
 #include "fft2.cuh"
 #include "fft_tc.cuh"
 #include "internal.h"
+#include "mix2.cuh"
 
 namespace scd {
 namespace {
@@ -268,6 +269,15 @@ const float2* table_pass_sym(int M, cudaError_t* err) {
 #undef SCD_PR
     default: *err = cudaErrorInvalidValue; return nullptr;
   }
+}
+
+// W_{L_s}^{k m} of every pass of a mixed-radix transform but the last (mix2.cuh), [k][m]
+const float2* table_mix(const MixPlan& plan, cudaError_t* err) {
+  return (const float2*)get_or_build(13, plan.P, 0, 0, sizeof(float2) * (size_t)plan.tw_len, err,
+                                     [&](void* p, cudaStream_t st) {
+    for (int s = 0; s + 1 < plan.n; ++s)
+      k_pass2<<<grid_for(plan.len[s]), 256, 0, st>>>((float2*)p + plan.off[s], plan.len[s + 1], plan.r[s]);
+  });
 }
 
 const float2* table_cols(int N, int M1, int C, cudaError_t* err) {

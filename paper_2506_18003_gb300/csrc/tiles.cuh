@@ -72,6 +72,19 @@ __host__ __device__ inline int64_t fam_pair_count(int Np, bool sym) {
   return sym ? (int64_t)Np * (Np + 1) / 2 : (int64_t)Np * Np;
 }
 
+// (kh, lh) of pair number `pair`: all Np^2, or (SYM) the folded triangle kh <= lh (fam_pairs_tile)
+template <bool SYM>
+__device__ __forceinline__ void fam_pair_of(int pair, int Np, int* kh, int* lh) {
+  if constexpr (SYM) {
+    const int r = pair / (Np + 1), c = pair - r * (Np + 1);
+    if (c < Np - r) { *kh = r; *lh = r + c; }
+    else { *kh = Np - 1 - r; *lh = c - 1; }
+  } else {
+    *kh = pair / Np;
+    *lh = pair - *kh * Np;
+  }
+}
+
 template <int PP, bool TC, bool PROF = false, bool SYM = false>
 __device__ __forceinline__ void fam_pairs_tile(float2* sm, TcCtx& ctx, const float2* __restrict__ X,
                                                const float2* __restrict__ Y, int Np, float2* __restrict__ out,
