@@ -70,7 +70,9 @@ typedef enum { SCD_FP32 = 0, SCD_SPLIT_BF16 = 1 } scd_precision;
  * AUTO: the choice scd_ssca_tune measured fastest for (N, Np, precision) on this GPU model
  *   (in this process, or from the SCD_TUNE_CACHE file); if never tuned, in the FP32 form the
  *   lag-domain kernels for an auto estimate of any power-of-two N, else FUSED where it fits,
- *   else STAGES. */
+ *   else STAGES.  An N that is not a power of two runs STAGES by Bluestein's identity, and under
+ *   AUTO in the FP32 form, where N is a product of two factors of radices 2 .. 16, mixed-radix
+ *   strip transforms. */
 typedef enum {
   SCD_SCHEDULE_AUTO = 0,
   SCD_SCHEDULE_STAGES = 1,
@@ -208,8 +210,8 @@ SCD_API scd_status scd_ssca_alpha_profile(const void* S, int64_t N, int32_t Np, 
 /* ------------------------------------------------------------------------------ batches
  * Batched form: nsig signals of uneven lengths through ONE persistent kernel launch (a
  * device work queue of per-signal stage tiles with bounded dependency waits), or the staged
- * schedule (one launch per stage and transform size over all signals; the default for SSCA
- * full estimates, see scd_batch_plan_set_schedule), captured in a CUDA graph that later runs
+ * schedule (one launch per stage and transform size over all signals; the default but for
+ * split-precision FAM plans, see scd_batch_plan_set_schedule), captured in a CUDA graph that later runs
  * with the same buffers and stream replay.
  *   estimator  0 = FAM (Np, L), 1 = SSCA (Np; L ignored)
  *   lengths    HOST array of nsig signal lengths (samples)
@@ -292,8 +294,9 @@ SCD_API scd_status scd_batch_plan_set_output(scd_batch_plan* plan, int32_t mode)
  * SCD_SCHEDULE_STAGES = one launch per stage and transform size over all signals (the
  * channelisers, then per size class the SSCA column passes in place on the workspace and row
  * passes, or the FAM pair transforms; same workspace, no device-side waits);
- * SCD_SCHEDULE_AUTO = the autotuner's choice for this workload, else the default of new plans
- * (STAGES for SSCA, PERSISTENT for FAM).  Both schedules serve both output modes. */
+ * SCD_SCHEDULE_AUTO = the autotuner's choice for this workload, else the default of new plans:
+ * one launch per stage and size class as well; in the FP32 form of the lag-domain SSCA kernels
+ * and the packed FAM pair transforms (split-precision FAM: PERSISTENT).  Both schedules serve both output modes. */
 SCD_API scd_status scd_batch_plan_set_schedule(scd_batch_plan* plan, int32_t schedule);
 
 /* ------------------------------------------------------------------------------ streaming
@@ -328,8 +331,8 @@ SCD_API scd_status scd_stream_advance(scd_batch_plan* plan, void* x_arena, const
  * from which later processes start.  Both calls enqueue and time real runs on `stream`
  * (the outputs hold a valid estimate afterwards) and synchronise it.
  *
- * scd_batch_tune: items of 32..512 KiB, SSCA slots of 8..64 MiB, and for full estimates the
- *   staged schedule; re-plans `plan` with the fastest setting (plans created later for the
+ * scd_batch_tune: items of 32..512 KiB, SSCA slots of 8..64 MiB, and the
+ *   staged schedules; re-plans `plan` with the fastest setting (plans created later for the
  *   same workload start from it).
  * scd_ssca_tune: the STAGES schedule and the PERSISTENT one with the same knobs, for
  *   (N, Np, opts->precision); later SCD_SCHEDULE_AUTO calls use the fastest.  Arguments as

@@ -182,18 +182,20 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
   }
   float2* ws = (float2*)o.workspace;
   if (!scd::is_pow2(N)) {
-    // any N: the strip transform on Bluestein's identity (staged kernels only)
+    // any N, staged kernels only: AUTO takes mixed-radix strips where N has a split (FP32); else, and under an
+    // explicit STAGES, which exact-length batch plans equal bit for bit, Bluestein's identity
+    const bool smooth = o.schedule == SCD_SCHEDULE_AUTO;
     if (o.schedule == SCD_SCHEDULE_PERSISTENT) return SCD_ERR_UNSUPPORTED;
     if (o.schedule != SCD_SCHEDULE_AUTO && o.schedule != SCD_SCHEDULE_STAGES && o.schedule != SCD_SCHEDULE_FUSED)
       return SCD_ERR_ARG;
     StageMarks m{o, 4};
     if ((e = m.mark(0, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_any_cdp((const float2*)x, y, conj, N, Np, window, ws, st, o.precision)) != cudaSuccess)
+    if ((e = scd::ssca_any_cdp((const float2*)x, y, conj, N, Np, window, ws, st, o.precision, smooth)) != cudaSuccess)
       return cuda_fail(e);
     if ((e = m.mark(1, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_any_first(N, Np, ws, st, o.precision)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_any_first(N, Np, ws, st, o.precision, smooth)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(2, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_any_second(N, Np, ws, (float2*)out, st, o.precision)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_any_second(N, Np, ws, (float2*)out, st, o.precision, smooth)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(3, st)) != cudaSuccess) return cuda_fail(e);
     return SCD_OK;
   }
@@ -367,7 +369,8 @@ scd_status scd_prepare(int32_t estimator, int64_t N, int32_t Np, int32_t P) {
         !scd::table_cols((int)M, M1, scd::ssca_cols_per_tile(M1), &e) || !scd::device_error_word(&e))
       return cuda_fail(e);
     if (scd::is_pow2(N) && !scd::ssca_lag_tables(N, Np, &e)) return cuda_fail(e);
-    if (!scd::is_pow2(N) && (!scd::table_chirp(N, &e) || !scd::table_bluestein_rows(N, M, M1, &e)))
+    if (!scd::is_pow2(N) && (!scd::table_chirp(N, &e) || !scd::table_bluestein_rows(N, M, M1, &e) ||
+                              !scd::prepare_strip(N, &e)))
       return cuda_fail(e);
     return SCD_OK;
   }

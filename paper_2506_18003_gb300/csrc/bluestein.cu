@@ -1,6 +1,8 @@
 // Kernels of the any-length DFTs (bluestein.cuh): the FAM pair stage for any P and the SSCA
 // strip transform for any N, in the FP32 form and the split-precision tensor-core form.
 //
+// FAM in the FP32 form runs mix2.cuh where P has a plan, else bluestein2.cuh for cyclic lengths 64 .. 4096; what
+// follows is the split-precision form and the lengths outside.
 // FAM (Eq. II.B-SCD_function_FAM with P not a power of two): one CTA runs C pairs; each pair's
 // conjugate product times the chirp goes through a size-MM FFT, the product with the kernel
 // spectrum stays in the transform's shared-memory region, a second FFT and the chirp give the
@@ -15,6 +17,8 @@
 //   1. the first size-M transform's column pass (reading the short rows, zero beyond), then the
 //      fused middle pass (row DFT, times Bh and conjugated, the second transform's row DFT);
 //   2. the second transform's column pass, c[j] conj(G[j]) for j < N stored fftshifted.
+// In the FP32 form a length that splits into two mixed-radix factors needs no chirp: stage 0 without it, then the
+// column pass W2 -> W1 and the row pass W1 -> output of mix2.cuh (N = 100,000, Np = 128: 407 -> 171 us).
 // Workspace: [x padded | y' padded | W1 (Np M) | W2 (Np M)]; X_g lives in W2 (row stride
 // Npad) until the middle pass overwrites it.
 #include <algorithm>
@@ -122,7 +126,7 @@ cudaError_t launch_fam_any2(const float2* X, const float2* Y, int Np, int P, flo
 
 // ---------------------------------------------------------------- SSCA
 // xp[n] = x[n], yp[n] = y[n] conj(c[n]) (conj: y[n] c[n]) for n < N, both 0 for N <= n < Npad.
-// The channeliser's product X_T conj(yp) (X_T yp) is then X_g(n, k) c[n].
+// (without a chirp yp = y.)  The channeliser's product X_T conj(yp) (X_T yp) is then X_g(n, k) c[n].
 __global__ void __launch_bounds__(256)
 k_bl_prep(const float2* __restrict__ x, const float2* __restrict__ y, int conj, int64_t N, int64_t Npad,
           const float2* __restrict__ chirp, float2* __restrict__ xp, float2* __restrict__ yp) {
@@ -130,8 +134,8 @@ k_bl_prep(const float2* __restrict__ x, const float2* __restrict__ y, int conj, 
     float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
     if (n < N) {
       a = __ldg(x + n);
-      const float2 yn = __ldg(y + n), cn = __ldg(chirp + n);
-      b = conj ? cmul(yn, cn) : cmulc(yn, cn);
+      b = __ldg(y + n);
+      if (chirp) b = conj ? cmul(b, __ldg(chirp + n)) : cmulc(b, __ldg(chirp + n));
     }
     xp[n] = a;
     yp[n] = b;
@@ -320,11 +324,12 @@ size_t ssca_any_workspace(int64_t N, int Np) {
 }
 
 cudaError_t ssca_any_cdp(const float2* x, const float2* y, bool conj, int64_t N, int Np, const float* window,
-                         void* ws, cudaStream_t st, int precision) {
+                         void* ws, cudaStream_t st, int precision, bool smooth) {
   const AnyLayout a = any_layout(N, Np, ws);
   cudaError_t err;
-  const float2* chirp = table_chirp(N, &err);
-  if (!chirp) return err;
+  StripPlan plan;
+  const float2* chirp = nullptr;
+  if ((!smooth || precision == SCD_SPLIT_BF16 || !strip_plan(N, &plan)) && !(chirp = table_chirp(N, &err))) return err;
   count_launches(1);
   k_bl_prep<<<(unsigned)std::min<int64_t>((a.Npad + 255) / 256, 152 * 8), 256, 0, st>>>(x, y, conj ? 1 : 0, N, a.Npad,
                                                                                       chirp, a.xp, a.yp);
@@ -332,9 +337,14 @@ cudaError_t ssca_any_cdp(const float2* x, const float2* y, bool conj, int64_t N,
   return ssca_cdp(a.xp, a.yp, conj, a.Npad, Np, window, a.w2, st, precision);
 }
 
-cudaError_t ssca_any_first(int64_t N, int Np, void* ws, cudaStream_t st, int precision) {
+cudaError_t ssca_any_first(int64_t N, int Np, void* ws, cudaStream_t st, int precision, bool smooth) {
   const AnyLayout a = any_layout(N, Np, ws);
   const bool tc = precision == SCD_SPLIT_BF16;
+  StripPlan plan;
+  if (smooth && !tc && strip_plan(N, &plan)) {                           // no chirp: the strips' column pass, X_g -> W1
+    count_launches(1);
+    return strip_cols(plan, N, Np, a.w2, a.Npad, a.w1, N, st);
+  }
   count_launches(2);
   // first transform's column pass: X_g (rows of Npad values) -> W1; fused middle: W1 -> W2
   cudaError_t err = tc ? launch_cols<true, false>(a.w2, a.Npad, a.Npad, a.w1, a.M, a.M, N, Np, a.M1, a.M2, nullptr, st)
@@ -344,13 +354,15 @@ cudaError_t ssca_any_first(int64_t N, int Np, void* ws, cudaStream_t st, int pre
             : launch_mid<false>(a.w1, a.w2, a.M, N, Np, a.M1, a.M2, st);
 }
 
-cudaError_t ssca_any_second(int64_t N, int Np, void* ws, float2* out, cudaStream_t st, int precision) {
+cudaError_t ssca_any_second(int64_t N, int Np, void* ws, float2* out, cudaStream_t st, int precision, bool smooth) {
   const AnyLayout a = any_layout(N, Np, ws);
+  const bool tc = precision == SCD_SPLIT_BF16;
+  StripPlan plan;
+  count_launches(1);
+  if (smooth && !tc && strip_plan(N, &plan)) return strip_rows(plan, N, Np, a.w1, N, out, N, st);
   cudaError_t err;
   const float2* chirp = table_chirp(N, &err);
   if (!chirp) return err;
-  const bool tc = precision == SCD_SPLIT_BF16;
-  count_launches(1);
   // second transform's column pass: W2 -> the fftshifted output (rows of N values)
   return tc ? launch_cols<true, true>(a.w2, a.M, a.M, out, N, a.M, N, Np, a.M1, a.M2, chirp, st)
             : launch_cols<false, true>(a.w2, a.M, a.M, out, N, a.M, N, Np, a.M1, a.M2, chirp, st);

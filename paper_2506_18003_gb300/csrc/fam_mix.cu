@@ -1,4 +1,4 @@
-// Launch of the mixed-radix FAM pair transforms (mix2.cuh).
+// Plans and launches of the mixed-radix FAM pair transforms and SSCA strips (mix2.cuh).
 #include <algorithm>
 
 #include "internal.h"
@@ -20,6 +20,20 @@ k_fam_mix(const __grid_constant__ MixPlan plan, int C, const float2* __restrict_
 
 // (Radices of at most 12 for three blocks per SM at 80 registers: within 3% at Np = 256, P = 500 and 1000,
 // slower where a further pass is needed: Np = 64, P = 1500 20.6 -> 26.6 us.)
+__global__ void __launch_bounds__(kMixThreads, kMixCtas)
+k_mix_cols(const __grid_constant__ MixPlan plan, const __grid_constant__ StripArgs A, const float2* __restrict__ in,
+           float2* __restrict__ out, const float2* __restrict__ tw, const float2* __restrict__ wN,
+           const float2* __restrict__ cols) {
+  extern __shared__ __align__(128) unsigned char mix_sm[];
+  mix_cols_cta(mix_sm, plan, A, in, out, tw, wN, cols);
+}
+__global__ void __launch_bounds__(kMixThreads, kMixCtas)
+k_mix_rows(const __grid_constant__ MixPlan plan, const __grid_constant__ StripArgs A, const float2* __restrict__ in,
+           float2* __restrict__ out, const float2* __restrict__ tw) {
+  extern __shared__ __align__(128) unsigned char mix_sm[];
+  mix_rows_cta(mix_sm, plan, A, in, out, tw);
+}
+
 // The non-increasing radices with the smallest sum whose product is P, n of them (0: none).
 int best_radices(int P, int n, int from, int* r) {
   if (n == 0) return P == 1 ? 0 : -1;
@@ -38,8 +52,10 @@ int best_radices(int P, int n, int from, int* r) {
 
 }  // namespace
 
-bool mix_plan(int P, MixPlan* p) {
-  if (P <= 16 || P > 4096 || is_pow2(P)) return false;         // 4096: one unit's values and twiddles in 113 KB
+bool mix_plan(int P, MixPlan* p) { return !is_pow2(P) && mix_factor(P, p); }
+
+bool mix_factor(int P, MixPlan* p) {
+  if (P <= 16 || P > 4096) return false;                       // 4096: one unit's values and twiddles in 113 KB
   p->n = 0;
   for (int n = 2; n <= 4 && !p->n; ++n)                        // as few passes as the radices allow
     if (best_radices(P, n, 0, p->r) > 0) p->n = n;
@@ -57,7 +73,7 @@ bool mix_plan(int P, MixPlan* p) {
   p->r0.set(p->r[0]);
   p->r1.set(p->r[1]);
   p->stride = p->len[1] | 1;
-  p->unit = p->r[0] * p->stride;
+  p->unit = (p->r[0] * p->stride) | 1;                         // odd too, for interleaved transforms
   return true;
 }
 
@@ -99,6 +115,87 @@ cudaError_t fam_mix_pairs(const float2* X, const float2* Y, int Np, const MixPla
   count_launches(1);
   return launch_dependent(true, sym ? k_fam_mix<true> : k_fam_mix<false>, grid, kMixThreads, mix_smem(plan, C), st, plan, C,
                           X, Y, Np, out, tw);
+}
+
+// ---------------------------------------------------------------- SSCA strips
+// Lane pairs per tile: up to 16, so that a tile's rows are contiguous runs of 256 bytes.
+static int strip_width(const MixPlan& p) {
+  int lc = 4;
+  while (lc > 0 && mix_smem(p, 1 << lc) > 112 * 1024) --lc;
+  return lc;
+}
+
+// Both factors with a plan (found once per length and thread); the widest tiles, then the fewest passes, then the smallest radix sum.
+static bool find_strip_plan(int64_t N, StripPlan* best) {
+  int64_t score = -1;
+  if (N > (int64_t)4096 * 4096 || N > INT32_MAX / 2) return false;
+  for (int64_t d = 17; d <= 4096 && d <= N / 17; ++d) {
+    StripPlan p;
+    if (N % d || N / d > 4096 || !mix_factor((int)d, &p.a) || !mix_factor((int)(N / d), &p.b)) continue;
+    p.N1 = (int)d;
+    p.N2 = (int)(N / d);
+    p.lca = strip_width(p.a);
+    p.lcb = strip_width(p.b);
+    int sum = 0;
+    for (int s = 0; s < p.a.n; ++s) sum += p.a.r[s];
+    for (int s = 0; s < p.b.n; ++s) sum += p.b.r[s];
+    const int odd = N % 4 == 0 && (p.N1 % 2 || p.N2 % 2);      // 16-byte accesses in both passes if N allows them
+    const int64_t v = ((int64_t)(p.lca < p.lcb ? p.lca : p.lcb) << 32) - ((int64_t)odd << 24) - ((p.a.n + p.b.n) << 16) - sum;
+    if (score < 0 || v > score) { score = v; *best = p; }
+  }
+  return score >= 0;
+}
+
+bool strip_plan(int64_t N, StripPlan* plan) {
+  thread_local int64_t last = 0;
+  thread_local bool found = false;
+  thread_local StripPlan kept;
+  if (last != N) {
+    found = find_strip_plan(N, &kept);
+    last = N;
+  }
+  if (found) *plan = kept;
+  return found;
+}
+
+bool prepare_strip(int64_t N, cudaError_t* err) {
+  StripPlan plan;
+  return !strip_plan(N, &plan) || (table_mix(plan.a, err) && table_mix(plan.b, err) && table_roots((int)N, err) &&
+                                   table_cols((int)N, plan.N1, 2 << plan.lca, err));
+}
+
+cudaError_t strip_cols(const StripPlan& plan, int64_t N, int rows, const float2* in, int64_t ld, float2* out, int64_t ldo,
+                       cudaStream_t st) {
+  cudaError_t err;
+  const int C = 1 << plan.lca;
+  const float2* tw = table_mix(plan.a, &err);
+  if (!tw) return err;
+  const float2* wN = table_roots((int)N, &err);
+  if (!wN) return err;
+  const float2* cols = table_cols((int)N, plan.N1, 2 * C, &err);
+  if (!cols) return err;
+  const int sms = sm_count(&err);
+  if (!sms) return err;
+  if ((err = allow_smem<k_mix_cols>(113 * 1024)) != cudaSuccess) return err;
+  StripArgs A{ld, ldo, plan.N1, plan.N2, (int)N, rows, plan.lca};
+  const int64_t tiles = (int64_t)(((plan.N2 + 1) / 2 + C - 1) / C) * rows;
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, kMixCtas * sms);
+  return launch_dependent(true, k_mix_cols, grid, kMixThreads, mix_smem(plan.a, C), st, plan.a, A, in, out, tw, wN, cols);
+}
+
+cudaError_t strip_rows(const StripPlan& plan, int64_t N, int rows, const float2* in, int64_t ld, float2* out, int64_t ldo,
+                       cudaStream_t st) {
+  cudaError_t err;
+  const int C = 1 << plan.lcb;
+  const float2* tw = table_mix(plan.b, &err);
+  if (!tw) return err;
+  const int sms = sm_count(&err);
+  if (!sms) return err;
+  if ((err = allow_smem<k_mix_rows>(113 * 1024)) != cudaSuccess) return err;
+  StripArgs A{ld, ldo, plan.N1, plan.N2, (int)N, rows, plan.lcb};
+  const int64_t tiles = (int64_t)(((plan.N1 + 1) / 2 + C - 1) / C) * rows;
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, kMixCtas * sms);
+  return launch_dependent(true, k_mix_rows, grid, kMixThreads, mix_smem(plan.b, C), st, plan.b, A, in, out, tw);
 }
 
 }  // namespace scd

@@ -22,6 +22,7 @@ const float2* table_pass2(int M, cudaError_t* err);        // ... of a paired si
 const float2* table_pass_sym(int M, cudaError_t* err);     // ... with the plan PlanSym<M>
 struct MixPlan;
 const float2* table_mix(const MixPlan& plan, cudaError_t* err);   // mixed-radix twiddles (mix2.cuh)
+bool prepare_strip(int64_t N, cudaError_t* err);           // ... of SSCA strips of N, if it has such a split
 bool prepare_mix(int P, cudaError_t* err);                 // ... built if P has such a plan
 const float2* table_cols(int N, int M1, int C, cudaError_t* err);  // W_N^{c m1'}, [m1'][c], c < C
 const float* table_hamming(int Np, cudaError_t* err);      // default window, float32
@@ -104,11 +105,12 @@ cudaError_t fam_pair_fft_any(const float2* X, const float2* Y, int Np, int P, fl
 // workspace ws (ssca_any_workspace bytes): channeliser + CDP with the chirp folded into the
 // second factor; the first size-M transform times the kernel spectrum; the second transform
 // into the fftshifted output.
+// (smooth: mixed-radix strips instead where N has such a split, mix2.cuh)
 size_t ssca_any_workspace(int64_t N, int Np);
 cudaError_t ssca_any_cdp(const float2* x, const float2* y, bool conj, int64_t N, int Np, const float* window,
-                         void* ws, cudaStream_t st, int precision);
-cudaError_t ssca_any_first(int64_t N, int Np, void* ws, cudaStream_t st, int precision);
-cudaError_t ssca_any_second(int64_t N, int Np, void* ws, float2* out, cudaStream_t st, int precision);
+                         void* ws, cudaStream_t st, int precision, bool smooth);
+cudaError_t ssca_any_first(int64_t N, int Np, void* ws, cudaStream_t st, int precision, bool smooth);
+cudaError_t ssca_any_second(int64_t N, int Np, void* ws, float2* out, cudaStream_t st, int precision, bool smooth);
 
 // ---------------------------------------------------------------- maps (map.cu)
 cudaError_t fam_map(const float2* S, int Np, int L, int P, int power, bool conj, float* map, cudaStream_t st);

@@ -1,4 +1,5 @@
-// Mixed-radix transforms on the packed lanes: the FAM pair transform for a P of at most 4096 that is not a
+// Mixed-radix transforms on the packed lanes: the SSCA strips of a length that splits into two factors with
+// such a plan (17 .. 4096 each), and the FAM pair transform for a P of at most 4096 that is not a
 // power of two but a product of up to four radices 2 .. 16 (every P = 2^a 3^b 5^c 7^d with few exceptions),
 // FP32 form.  One transform of size P per pair, where Bluestein's identity (bluestein2.cuh) takes two of
 // size >= 2 P - 1.
@@ -154,8 +155,20 @@ struct MixPlan {
   Div16 per[4], m[4], r0, r1;                                  // P / r_s, L_{s+1}, r_0, r_1
 };
 
-// The plan of a length P (only its n, radices, lengths and table sizes depend on P); false: no plan.
+// The plan of any length 17 .. 4096 that is such a product (powers of two too); false: none.
+bool mix_factor(int P, MixPlan* plan);
+// The plan of a FAM length P (only its n, radices, lengths and table sizes depend on P); false: no plan.
 bool mix_plan(int P, MixPlan* plan);
+// SSCA strips of length N (FP32): the split N1 N2 and the tile widths; false: no split.
+struct StripPlan {
+  MixPlan a, b;                                                // the column pass (N1), the row pass (N2)
+  int N1, N2, lca, lcb;
+};
+bool strip_plan(int64_t N, StripPlan* plan);
+cudaError_t strip_cols(const StripPlan& plan, int64_t N, int rows, const float2* in, int64_t ld, float2* out, int64_t ldo,
+                       cudaStream_t st);
+cudaError_t strip_rows(const StripPlan& plan, int64_t N, int rows, const float2* in, int64_t ld, float2* out, int64_t ldo,
+                       cudaStream_t st);
 cudaError_t fam_mix_pairs(const float2* X, const float2* Y, int Np, const MixPlan& plan, float2* out, cudaStream_t st);
 
 constexpr int kMixThreads = 256, kMixCtas = 2, kMixMaxUnits = 16;
@@ -178,6 +191,98 @@ __device__ __forceinline__ void with_radix(int r, F&& f) {
     case 15: f(Radix<15>{}); break;
     case 16: f(Radix<16>{}); break;
   }
+}
+
+// The passes of one tile, cv transforms (of C, a power of two when CF) in the exchange area sm.  CF: neighbouring
+// threads take the same butterfly of neighbouring transforms (interleaved data), else neighbouring butterflies.
+// src(radix, c, m, step, v) gives v[j] = input m + j step of transform c; dst(radix, c, i, step, v) takes bins
+// i + j step.
+template <bool CF>
+__device__ __forceinline__ bool mix_split(int b, const Div16& per, int lc, int cv, int* c, int* i) {
+  if constexpr (CF) {
+    *c = b & ((1 << lc) - 1);
+    *i = b >> lc;
+    return *c < cv;
+  } else {
+    *c = (int)per.quot(b);
+    *i = b - *c * (int)per.d;
+    return true;
+  }
+}
+template <bool CF>
+__device__ __forceinline__ int mix_total(const Div16& per, int lc, int cv) {
+  return CF ? (int)per.d << lc : cv * (int)per.d;
+}
+
+template <bool CF, class Src>
+__device__ __forceinline__ void mix_first(float4* sm, const float2* tws, const MixPlan& pl, int lc, int cv, Src&& src) {
+  with_radix(pl.r[0], [&](auto rr) {
+    constexpr int R = decltype(rr)::r;
+    const int L1 = pl.len[1], total = mix_total<CF>(pl.per[0], lc, cv);
+    for (int b = threadIdx.x; b < total; b += kMixThreads) {
+      int c, m;
+      if (!mix_split<CF>(b, pl.per[0], lc, cv, &c, &m)) continue;
+      C2 v[R];
+      src(rr, c, m, L1, v);
+      dft_any<R>(v);
+      float4* d = sm + c * pl.unit + m;
+      d[0] = c2_f4(v[0]);
+#pragma unroll
+      for (int k = 1; k < R; ++k) d[k * pl.stride] = c2_f4(cmul(v[k], tws[k * L1 + m]));
+    }
+  });
+}
+
+template <bool CF>
+__device__ __forceinline__ void mix_middle(float4* sm, const float2* tws, const MixPlan& pl, int lc, int cv) {
+  for (int s = 1; s + 1 < pl.n; ++s) {
+    with_radix(pl.r[s], [&](auto rr) {
+      constexpr int R = decltype(rr)::r;
+      const int Ln = pl.len[s + 1], total = mix_total<CF>(pl.per[s], lc, cv);
+      const float2* w = tws + pl.off[s];
+      for (int b = threadIdx.x; b < total; b += kMixThreads) {
+        int c, i;
+        if (!mix_split<CF>(b, pl.per[s], lc, cv, &c, &i)) continue;
+        const int blk = (int)pl.m[s].quot(i), m = i - blk * Ln;
+        const int k0 = s == 1 ? blk : (int)pl.r1.quot(blk), rest = s == 1 ? 0 : (blk - k0 * pl.r[1]) * pl.len[2];
+        float4* d = sm + c * pl.unit + k0 * pl.stride + rest + m;
+        C2 v[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) v[j] = take2(d + j * Ln);
+        dft_any<R>(v);
+        d[0] = c2_f4(v[0]);
+#pragma unroll
+        for (int k = 1; k < R; ++k) d[k * Ln] = c2_f4(cmul(v[k], w[k * Ln + m]));
+      }
+    });
+    __syncthreads();
+  }
+}
+
+template <bool CF, class Dst>
+__device__ __forceinline__ void mix_last(const float4* sm, const MixPlan& pl, int lc, int cv, Dst&& dst) {
+  with_radix(pl.r[pl.n - 1], [&](auto rr) {
+    constexpr int R = decltype(rr)::r;
+    const Div16& per = pl.per[pl.n - 1];
+    const int total = mix_total<CF>(per, lc, cv);
+    for (int b = threadIdx.x; b < total; b += kMixThreads) {
+      int c, i;
+      if (!mix_split<CF>(b, per, lc, cv, &c, &i)) continue;
+      const int i1 = (int)pl.r0.quot(i), k0 = i - i1 * pl.r[0];
+      int at = k0 * pl.stride;
+      if (pl.n == 3) at += i1 * pl.len[2];
+      if (pl.n == 4) {
+        const int k2 = (int)pl.r1.quot(i1);
+        at += (i1 - k2 * pl.r[1]) * pl.len[2] + k2 * pl.len[3];
+      }
+      const float4* d = sm + c * pl.unit + at;
+      C2 v[R];
+#pragma unroll
+      for (int j = 0; j < R; ++j) v[j] = take2(d + j);
+      dft_any<R>(v);
+      dst(rr, c, i, (int)per.d, v);
+    }
+  });
 }
 
 // FAM pairs two by two, persistent over tiles of C units (one unit = two pairs; their number is even).
@@ -206,76 +311,141 @@ __device__ __forceinline__ void fam_mix_cta(unsigned char* smem, const MixPlan& 
                                   SYM && k1 != l1 ? (l1 * Np + k1) * P : -1);
     }
     __syncthreads();                                           // and every read of the last tile's values is done
-    with_radix(pl.r[0], [&](auto rr) {
+    mix_first<false>(sm, tws, pl, 0, cv, [&](auto rr, int c, int m, int L1, C2* v) {
       constexpr int R = decltype(rr)::r;
-      const int L1 = pl.len[1], total = cv * L1;
-      for (int b = tid; b < total; b += kMixThreads) {
-        const int c = (int)pl.per[0].quot(b), m = b - c * L1;
-        const int4 row = my[2 * c];
-        const float2 *a0 = X + row.x + m, *b0 = Y + row.y + m, *a1 = X + row.z + m, *b1 = Y + row.w + m;
-        C2 v[R];
+      const int4 row = my[2 * c];
+      const float2 *a0 = X + row.x + m, *b0 = Y + row.y + m, *a1 = X + row.z + m, *b1 = Y + row.w + m;
 #pragma unroll
-        for (int j = 0; j < R; ++j)
-          v[j] = c2_pack(cmulc(__ldg(a0 + j * L1), __ldg(b0 + j * L1)), cmulc(__ldg(a1 + j * L1), __ldg(b1 + j * L1)));
-        dft_any<R>(v);
-        float4* d = sm + c * pl.unit + m;
-        d[0] = c2_f4(v[0]);
+      for (int j = 0; j < R; ++j)
+        v[j] = c2_pack(cmulc(__ldg(a0 + j * L1), __ldg(b0 + j * L1)), cmulc(__ldg(a1 + j * L1), __ldg(b1 + j * L1)));
+    });
+    __syncthreads();
+    mix_middle<false>(sm, tws, pl, 0, cv);
+    mix_last<false>(sm, pl, 0, cv, [&](auto rr, int c, int i, int nb, const C2* v) {
+      constexpr int R = decltype(rr)::r;
+      const int4 o = my[2 * c + 1];
 #pragma unroll
-        for (int k = 1; k < R; ++k) d[k * pl.stride] = c2_f4(cmul(v[k], tws[k * L1 + m]));
+      for (int j = 0; j < R; ++j) {
+        const int f = i + nb * j;
+        const float2 s0 = c2_lane0(v[j]), s1 = c2_lane1(v[j]);
+        const int q = f + half < P ? f + half : f + half - P;
+        out[o.x + q] = s0;
+        out[o.y + q] = s1;
+        if constexpr (SYM) {
+          const int fm = f == 0 ? 0 : P - f, qm = fm + half < P ? fm + half : fm + half - P;
+          if (o.z >= 0) out[o.z + qm] = cconj(s0);
+          if (o.w >= 0) out[o.w + qm] = cconj(s1);
+        }
+      }
+    });
+  }
+}
+
+// ---------------------------------------------------------------- SSCA strips of length N = N1 N2
+// Two passes over Np N values, where Bluestein's identity takes three over Np M, M >= 2 N - 1, with twice the
+// transforms: N = 100,000 (250 x 400), Np = 128 takes 171 us instead of 407 (28 of them the channeliser in both).
+// Bound by the traffic between the passes, 102 MB written and read twice, most of it in L2, in runs of 256
+// bytes; 16 columns or row pairs per tile where they fit half an SM's shared memory.
+// Column pass: n = n1 N2 + n2, transforms over n1 of the columns n2, two columns per lane pair:
+//   out[k1 N2 + n2] = W_N^{n2 k1} sum_{n1} W_N1^{k1 n1} in[n1 N2 + n2],
+// in rows of stride ld, out rows of stride ldo (both even, 16-byte aligned).  The rotation is W_N^{n0 k1}
+// (table of roots) times W_N^{d k1} (`cols`, [k1][d], d < 2 C) for column n0 + d of a tile.
+struct StripArgs {
+  int64_t ld, ldo;
+  int N1, N2, N, rows, lc;                                     // rows: strips; C = 2^lc lane pairs per tile
+};
+
+__device__ __forceinline__ void mix_cols_cta(unsigned char* smem, const MixPlan& pl, const StripArgs& A,
+                                             const float2* __restrict__ in, float2* __restrict__ out,
+                                             const float2* __restrict__ tw, const float2* __restrict__ wN,
+                                             const float2* __restrict__ cols) {
+  const int C = 1 << A.lc, N2 = A.N2, tid = (int)threadIdx.x;
+  float4* sm = reinterpret_cast<float4*>(smem);
+  float2* tws = reinterpret_cast<float2*>(sm + C * pl.unit);
+  for (int e = tid; e < pl.tw_len; e += kMixThreads) tws[e] = __ldg(tw + e);
+  const int per_row = ((N2 + 1) / 2 + C - 1) / C, tiles = per_row * A.rows;
+  const bool even = N2 % 2 == 0;
+  wait_for_previous();
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (tile + (int)gridDim.x >= tiles) let_next_start();
+    const int row = tile / per_row, n0 = (tile - row * per_row) * 2 * C, cv = min(C, (N2 - n0 + 1) / 2);
+    const float2* src = in + row * A.ld + n0;
+    float2* dst = out + row * A.ldo + n0;
+    __syncthreads();
+    mix_first<true>(sm, tws, pl, A.lc, cv, [&](auto rr, int c, int m, int L1, C2* v) {
+      constexpr int R = decltype(rr)::r;
+      const float2* p = src + m * N2 + 2 * c;
+      const bool both = n0 + 2 * c + 1 < N2;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        if (even) {
+          const float4 q = __ldg(reinterpret_cast<const float4*>(p + j * L1 * N2));
+          v[j] = c2_pack(make_float2(q.x, q.y), make_float2(q.z, q.w));
+        } else {
+          v[j] = c2_pack(__ldg(p + j * L1 * N2), both ? __ldg(p + j * L1 * N2 + 1) : make_float2(0.f, 0.f));
+        }
       }
     });
     __syncthreads();
-    for (int s = 1; s + 1 < pl.n; ++s) {
-      with_radix(pl.r[s], [&](auto rr) {
-        constexpr int R = decltype(rr)::r;
-        const int Ln = pl.len[s + 1], nb = (int)pl.per[s].d, total = cv * nb;
-        const float2* w = tws + pl.off[s];
-        for (int b = tid; b < total; b += kMixThreads) {
-          const int c = (int)pl.per[s].quot(b), i = b - c * nb;
-          const int blk = (int)pl.m[s].quot(i), m = i - blk * Ln;
-          const int k0 = s == 1 ? blk : (int)pl.r1.quot(blk), rest = s == 1 ? 0 : (blk - k0 * pl.r[1]) * pl.len[2];
-          float4* d = sm + c * pl.unit + k0 * pl.stride + rest + m;
-          C2 v[R];
-#pragma unroll
-          for (int j = 0; j < R; ++j) v[j] = take2(d + j * Ln);
-          dft_any<R>(v);
-          d[0] = c2_f4(v[0]);
-#pragma unroll
-          for (int k = 1; k < R; ++k) d[k * Ln] = c2_f4(cmul(v[k], w[k * Ln + m]));
-        }
-      });
-      __syncthreads();
-    }
-    with_radix(pl.r[pl.n - 1], [&](auto rr) {
+    mix_middle<true>(sm, tws, pl, A.lc, cv);
+    mix_last<true>(sm, pl, A.lc, cv, [&](auto rr, int c, int i, int nb, const C2* v) {
       constexpr int R = decltype(rr)::r;
-      const int nb = (int)pl.per[pl.n - 1].d, total = cv * nb;
-      for (int b = tid; b < total; b += kMixThreads) {
-        const int c = (int)pl.per[pl.n - 1].quot(b), i = b - c * nb;
-        const int i1 = (int)pl.r0.quot(i), k0 = i - i1 * pl.r[0];
-        int at = k0 * pl.stride;
-        if (pl.n == 3) at += i1 * pl.len[2];
-        if (pl.n == 4) {
-          const int k2 = (int)pl.r1.quot(i1);
-          at += (i1 - k2 * pl.r[1]) * pl.len[2] + k2 * pl.len[3];
+      const bool both = n0 + 2 * c + 1 < N2;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const int k1 = i + nb * j;
+        const float4 w = __ldg(reinterpret_cast<const float4*>(cols + 2 * (k1 * C + c)));
+        const C2 g = cmul(cmul(v[j], C2{make_float2(w.x, w.z), make_float2(w.y, w.w)}), __ldg(wN + n0 * k1));
+        float2* p = dst + (int64_t)k1 * N2 + 2 * c;
+        if (even) {
+          *reinterpret_cast<float4*>(p) = make_float4(g.re.x, g.im.x, g.re.y, g.im.y);
+        } else {
+          p[0] = c2_lane0(g);
+          if (both) p[1] = c2_lane1(g);
         }
-        const float4* d = sm + c * pl.unit + at;
-        C2 v[R];
+      }
+    });
+  }
+}
+
+// Row pass: transforms over n2 of the rows k1, two rows per lane pair; bin q = k1 + N1 k2 goes to
+// out[(q + N / 2) mod N] of its strip.
+__device__ __forceinline__ void mix_rows_cta(unsigned char* smem, const MixPlan& pl, const StripArgs& A,
+                                             const float2* __restrict__ in, float2* __restrict__ out,
+                                             const float2* __restrict__ tw) {
+  const int C = 1 << A.lc, N1 = A.N1, N2 = A.N2, N = A.N, half = N / 2, tid = (int)threadIdx.x;
+  float4* sm = reinterpret_cast<float4*>(smem);
+  float2* tws = reinterpret_cast<float2*>(sm + C * pl.unit);
+  for (int e = tid; e < pl.tw_len; e += kMixThreads) tws[e] = __ldg(tw + e);
+  const int per_row = ((N1 + 1) / 2 + C - 1) / C, tiles = per_row * A.rows;
+  const bool even = N1 % 2 == 0 && N % 4 == 0;                 // two bins then are one aligned 16-byte store
+  wait_for_previous();
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (tile + (int)gridDim.x >= tiles) let_next_start();
+    const int row = tile / per_row, r0 = (tile - row * per_row) * 2 * C, cv = min(C, (N1 - r0 + 1) / 2);
+    const float2* src = in + row * A.ld + (int64_t)r0 * N2;
+    float2* dst = out + row * A.ldo;
+    __syncthreads();
+    mix_first<false>(sm, tws, pl, 0, cv, [&](auto rr, int c, int m, int L1, C2* v) {
+      constexpr int R = decltype(rr)::r;
+      const float2* p0 = src + 2 * c * N2 + m;
+      const float2* p1 = r0 + 2 * c + 1 < N1 ? p0 + N2 : p0;
 #pragma unroll
-        for (int j = 0; j < R; ++j) v[j] = take2(d + j);
-        dft_any<R>(v);
-        const int4 o = my[2 * c + 1];
+      for (int j = 0; j < R; ++j) v[j] = c2_pack(__ldg(p0 + j * L1), __ldg(p1 + j * L1));
+    });
+    __syncthreads();
+    mix_middle<false>(sm, tws, pl, 0, cv);
+    mix_last<true>(sm, pl, A.lc, cv, [&](auto rr, int c, int i, int nb, const C2* v) {
+      constexpr int R = decltype(rr)::r;
+      const int k1 = r0 + 2 * c;
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-          const int f = i + nb * j;
-          const float2 s0 = c2_lane0(v[j]), s1 = c2_lane1(v[j]);
-          const int q = f + half < P ? f + half : f + half - P;
-          out[o.x + q] = s0;
-          out[o.y + q] = s1;
-          if constexpr (SYM) {
-            const int fm = f == 0 ? 0 : P - f, qm = fm + half < P ? fm + half : fm + half - P;
-            if (o.z >= 0) out[o.z + qm] = cconj(s0);
-            if (o.w >= 0) out[o.w + qm] = cconj(s1);
-          }
+      for (int j = 0; j < R; ++j) {
+        const int q = k1 + N1 * (i + nb * j), at = q + half < N ? q + half : q + half - N;
+        if (even) {
+          *reinterpret_cast<float4*>(dst + at) = make_float4(v[j].re.x, v[j].im.x, v[j].re.y, v[j].im.y);
+        } else {
+          dst[at] = c2_lane0(v[j]);
+          if (k1 + 1 < N1) dst[at + 1 < N ? at + 1 : 0] = c2_lane1(v[j]);
         }
       }
     });
