@@ -1,6 +1,7 @@
 // Batched form: hundreds of signals of uneven lengths through one CUDA graph per estimator,
 // holding either ONE persistent launch (below) or the staged schedule's launches (one per
-// stage and size class, batch_staged.cu; the SSCA default).
+// stage and size class, batch_staged.cu; the default but for split-precision FAM plans; FP32 plans then run
+// the lag-domain SSCA (ssca_lag.cuh) and the packed FAM pair transforms (fam2.cuh) per size class).
 //
 // A batch plan lists tasks (one stage of one signal: FAM channeliser / pair FFT, SSCA
 // channeliser+CDP / column pass / row pass), each a range of tiles (one tile = one CTA's
