@@ -870,7 +870,7 @@ def measure_variants(torch, binding, dev, stream, reps=10, warmup=2):
     pf = torch.empty(2 * P * L, dtype=torch.float32, device=dev)
     ps = torch.empty(2 * Ns, dtype=torch.float32, device=dev)
     lib = binding.load()
-    # lengths that are not powers of two (Bluestein's identity): FAM P = 1000, SSCA N = 500,000
+    # lengths that are not powers of two: FAM P = 1000, SSCA N = 500,000
     Pa, Na = 1000, 500000
     work = torch.empty(max(lib.scd_fam_workspace_bytes(Nf, Np, L, P, 0), lib.scd_ssca_workspace_bytes(Ns, Nps, 0),
                            lib.scd_fam_workspace_bytes(Nf, Np, L, Pa, 0), lib.scd_ssca_workspace_bytes(Na, Nps, 0)),
@@ -916,7 +916,7 @@ def measure_variants(torch, binding, dev, stream, reps=10, warmup=2):
     torch.cuda.empty_cache()
     out["paper_match"] = paper_match(torch, binding, dev, stream, reps)
     out["sizes"] = ("FAM N=65728 Np=256 L=64 P=1024; SSCA N=2^20 Np=256; any-length: FAM P=1000 (N=64,192), "
-                    "SSCA N=500,000 (Bluestein, cyclic length 2^20); FP32 form; %d calls each" % reps)
+                    "SSCA N=500,000; FP32 form; %d calls each" % reps)
     # streaming: one group of windows per step, new samples copied in from pinned host memory
     # every step (scd_stream_advance) and the plan's graph replayed (scd_batch_run)
     for name, est, W, hop, nwin, Npw, Lw in (("ssca_stream", "ssca", 1 << 16, 1 << 15, 16, 256, 1),

@@ -344,8 +344,9 @@ __device__ __forceinline__ void fam_mix_cta(unsigned char* smem, const MixPlan& 
 // ---------------------------------------------------------------- SSCA strips of length N = N1 N2
 // Two passes over Np N values, where Bluestein's identity takes three over Np M, M >= 2 N - 1, with twice the
 // transforms: N = 100,000 (250 x 400), Np = 128 takes 171 us instead of 407 (28 of them the channeliser in both).
-// Bound by the traffic between the passes, 102 MB written and read twice, most of it in L2, in runs of 256
-// bytes; 16 columns or row pairs per tile where they fit half an SM's shared memory.
+// Bound by latency: 16 warps per SM at 0.3 of the issue slots, waiting on the tile's loads and at the barriers
+// between its phases (76 and 65 us cold, 2 TB/s of DRAM traffic).  16 columns or row pairs per tile where they
+// fit half an SM's shared memory, so that both passes read or write runs of 256 bytes.
 // Column pass: n = n1 N2 + n2, transforms over n1 of the columns n2, two columns per lane pair:
 //   out[k1 N2 + n2] = W_N^{n2 k1} sum_{n1} W_N1^{k1 n1} in[n1 N2 + n2],
 // in rows of stride ld, out rows of stride ldo (both even, 16-byte aligned).  The rotation is W_N^{n0 k1}
