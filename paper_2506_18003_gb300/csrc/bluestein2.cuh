@@ -70,7 +70,8 @@ __device__ __forceinline__ void fam_any2_cta(unsigned char* smem, const float2* 
       for (int r = 0; r < E / 2; ++r) {
         const int p = t + r * T;
         if (p < P)
-          v[r] = cmul(c2_pack(cmulc(__ldg(a0 + p), __ldg(b0 + p)), cmulc(__ldg(a1 + p), __ldg(b1 + p))), __ldg(chirp + p));
+          v[r] = cmul(c2_pack(cmulc(load_written(a0 + p), load_written(b0 + p)), cmulc(load_written(a1 + p), load_written(b1 + p))),
+                      __ldg(chirp + p));
         else
           v[r] = C2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
       }

@@ -30,8 +30,8 @@ k_fam_channelise(const float2* __restrict__ x, int L, int P, const float* __rest
   using FS = FftSmem<NP, S::C, S::NT, TC>;
   unsigned char* base = reinterpret_cast<unsigned char*>(sm);
   if constexpr (!TC) {
-    let_next_start();
     wait_for_previous();
+    let_next_start();
   }
   TcCtx ctx{};
   if constexpr (TC) ctx = tc_begin<FS::tmem_cols>(base + FS::region0 + FS::bbytes, base + FS::region0, bmats, FS::bbytes, err);
@@ -50,8 +50,8 @@ __device__ __forceinline__ void fam_pairs_cta(const float2* __restrict__ X, cons
   using FS = FftSmem<PP, S::C, S::NT, TC>;
   unsigned char* base = reinterpret_cast<unsigned char*>(sm);
   if constexpr (!TC) {
-    let_next_start();
     wait_for_previous();
+    let_next_start();
   }
   TcCtx ctx{};
   if constexpr (TC) ctx = tc_begin<FS::tmem_cols>(base + FS::region0 + FS::bbytes, base + FS::region0, bmats, FS::bbytes, err);

@@ -95,7 +95,7 @@ __device__ __forceinline__ void fam_pairs2_cta(unsigned char* sm, const FamArgs&
     C2 v[E];
 #pragma unroll
     for (int r = 0; r < E; ++r) {
-      const float4 a = __ldg(xk + r * (M / E)), b = __ldg(yl + r * (M / E));
+      const float4 a = load_written(xk + r * (M / E)), b = load_written(yl + r * (M / E));
       v[r] = c2_pack(cmulc(make_float2(a.x, a.y), make_float2(b.x, b.y)),
                      cmulc(make_float2(a.z, a.w), make_float2(b.z, b.w)));
     }

@@ -317,7 +317,8 @@ __device__ __forceinline__ void fam_mix_cta(unsigned char* smem, const MixPlan& 
       const float2 *a0 = X + row.x + m, *b0 = Y + row.y + m, *a1 = X + row.z + m, *b1 = Y + row.w + m;
 #pragma unroll
       for (int j = 0; j < R; ++j)
-        v[j] = c2_pack(cmulc(__ldg(a0 + j * L1), __ldg(b0 + j * L1)), cmulc(__ldg(a1 + j * L1), __ldg(b1 + j * L1)));
+        v[j] = c2_pack(cmulc(load_written(a0 + j * L1), load_written(b0 + j * L1)),
+                       cmulc(load_written(a1 + j * L1), load_written(b1 + j * L1)));
     });
     __syncthreads();
     mix_middle<false>(sm, tws, pl, 0, cv);
@@ -380,10 +381,10 @@ __device__ __forceinline__ void mix_cols_cta(unsigned char* smem, const MixPlan&
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         if (even) {
-          const float4 q = __ldg(reinterpret_cast<const float4*>(p + j * L1 * N2));
+          const float4 q = load_written(reinterpret_cast<const float4*>(p + j * L1 * N2));
           v[j] = c2_pack(make_float2(q.x, q.y), make_float2(q.z, q.w));
         } else {
-          v[j] = c2_pack(__ldg(p + j * L1 * N2), both ? __ldg(p + j * L1 * N2 + 1) : make_float2(0.f, 0.f));
+          v[j] = c2_pack(load_written(p + j * L1 * N2), both ? load_written(p + j * L1 * N2 + 1) : make_float2(0.f, 0.f));
         }
       }
     });
@@ -432,7 +433,7 @@ __device__ __forceinline__ void mix_rows_cta(unsigned char* smem, const MixPlan&
       const float2* p0 = src + 2 * c * N2 + m;
       const float2* p1 = r0 + 2 * c + 1 < N1 ? p0 + N2 : p0;
 #pragma unroll
-      for (int j = 0; j < R; ++j) v[j] = c2_pack(__ldg(p0 + j * L1), __ldg(p1 + j * L1));
+      for (int j = 0; j < R; ++j) v[j] = c2_pack(load_written(p0 + j * L1), load_written(p1 + j * L1));
     });
     __syncthreads();
     mix_middle<false>(sm, tws, pl, 0, cv);

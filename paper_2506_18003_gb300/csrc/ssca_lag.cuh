@@ -176,15 +176,15 @@ __device__ __forceinline__ void lag_cols_tile(unsigned char* sm, const LagArgs& 
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int n = r * (M1 / E) * M2;
-    const float2 a = __ldg(xp + n);
+    const float2 a = load_written(xp + n);
     float2 b0, b1;
     if (r < E - 1) {                                        // n + m + 1 < N: the lags are far below N / E
-      b0 = __ldg(xp + n + m);
-      b1 = __ldg(xp + n + m + 1);
+      b0 = load_written(xp + n + m);
+      b1 = load_written(xp + n + m + 1);
     } else {
       const int nn = n + t * M2 + m2 + m;
-      b0 = nn < N ? __ldg(xp + n + m) : make_float2(0.f, 0.f);
-      b1 = nn + 1 < N ? __ldg(xp + n + m + 1) : make_float2(0.f, 0.f);
+      b0 = nn < N ? load_written(xp + n + m) : make_float2(0.f, 0.f);
+      b1 = nn + 1 < N ? load_written(xp + n + m + 1) : make_float2(0.f, 0.f);
     }
     v[r] = c2_pack(cmulc(b0, a), cmulc(b1, a));
   }
@@ -335,7 +335,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
       for (int i = 0; i < E / 2; ++i) {
         float2 r0 = neg[-i * S0 * K::neg_row];
         const float2 r1 = neg[-i * S0 * K::neg_row - 1];
-        if (wrap) r0 = __ldg(r0p - i * S0 * N);
+        if (wrap) r0 = load_written(r0p - i * S0 * N);
         const C2 f = cmul(i ? cmul(u, take2(step + i * C + c)) : u, turn[mh - 1 - i * S0]);
         v[E / 2 + i] = c2_pack(cmulc(c2_lane0(f), r0), cmulc(c2_lane1(f), r1));
       }

@@ -4,6 +4,7 @@
 // and C = THREADS / T transforms, in the FP32 form or (TC) the split tensor-core form.
 #pragma once
 #include "fft_tc.cuh"
+#include "pdl.cuh"
 
 namespace scd {
 
@@ -14,6 +15,14 @@ struct TileShape {
   static constexpr int C = T >= THREADS ? 1 : THREADS / T;
   static constexpr int NT = C * T;                      // threads actually used
 };
+
+// What an earlier kernel of the stream may have written (pdl.cuh); the split form's kernels are launched the
+// ordinary way, after that kernel's end, and keep the read-only path.
+template <bool TC, class T>
+__device__ __forceinline__ T load_input(const T* p) {
+  if constexpr (TC) return __ldg(p);
+  else return load_written(p);
+}
 
 // prof[i] = max(prof[i], v) for a non-negative float given by its bits (non-negative floats
 // order like their bit patterns); a fire-and-forget reduction in L2.  (Reading the current
@@ -43,7 +52,7 @@ __device__ __forceinline__ void fam_channelise_tile(float2* sm, TcCtx& ctx, cons
     const int p = p0 + c;
     if (p >= P) return make_float2(0.f, 0.f);
     const int n = (j - (int)(((int64_t)p * L) & (NP - 1))) & (NP - 1);    // j = (pL + n) mod Np
-    return cscale(__ldg(x + (int64_t)p * L + n), __ldg(a + n));
+    return cscale(load_input<TC>(x + (int64_t)p * L + n), load_input<TC>(a + n));
   };
   auto dst = [&](int c, int f, float2 v) {
     const int p = p0 + c;
@@ -111,7 +120,7 @@ __device__ __forceinline__ void fam_pairs_tile(float2* sm, TcCtx& ctx, const flo
   float2* __restrict__ o = PROF ? nullptr : out + ((int64_t)kh * Np + lh) * PP;
   float2* __restrict__ om = PROF ? nullptr : out + ((int64_t)lh * Np + kh) * PP;
   auto src = [&](int, int p) -> float2 {
-    return valid ? cmulc(__ldg(xk + p), __ldg(xl + p)) : make_float2(0.f, 0.f);
+    return valid ? cmulc(load_input<TC>(xk + p), load_input<TC>(xl + p)) : make_float2(0.f, 0.f);
   };
   auto dst = [&](int, int f, float2 v) {
     if constexpr (PROF) {
