@@ -285,6 +285,8 @@ SCD_API scd_status scd_host_free(void* ptr);
  * alpha profile of |S| / |S|^2 (scd_fam_alpha_profile / scd_ssca_alpha_profile of its
  * estimate, bit for bit), reduced inside the last stage so the estimate is never written
  * (the output shrinks from Np^2 P_i or Np N_i complex values to 2 P_i L or 2 N_i floats).
+ * A signal with a NaN sample gets NaN in every column that one of its NaN bins falls on, under every
+ * schedule (scd_*_alpha_profile of a stored estimate passes over NaN bins instead).
  * Changes the layout: scd_batch_query then gives out_offsets in float32 elements and the
  * out arena is float32[out_offsets[nsig]], zeroed by every run.  FAM needs 2 L <= Np and
  * P_i L divisible by Np for every signal (else SCD_ERR_UNSUPPORTED). */

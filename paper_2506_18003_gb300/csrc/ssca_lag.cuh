@@ -353,16 +353,17 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
     if constexpr (PROF) {
       // S(k, q) with k D + q = c mod N (q in [-N/2, N/2)) lies on alpha column c + N if k D + q = c, on
       // column c if it is c - N
-      float best[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+      // (maxima of the bits, as profile_max takes them: a NaN bin makes its column NaN, where fmaxf drops it)
+      unsigned best[2][2] = {{0u, 0u}, {0u, 0u}};
       auto dst = [&](int, int, int f, const C2& val) {
         const int k = ((f + H) & (NP - 1)) - H;
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
           const float2 s = l ? c2_lane1(val) : c2_lane0(val);
-          const float m2 = fmaf(s.x, s.x, s.y * s.y);
-          float* b = best[l];                               // q = f0 + l - k D, less N if that is >= N/2
-          if (f0 + l - k * D < N / 2) b[1] = fmaxf(b[1], m2);
-          else b[0] = fmaxf(b[0], m2);
+          const unsigned m2 = __float_as_uint(fmaf(s.x, s.x, s.y * s.y));
+          unsigned* b = best[l];                               // q = f0 + l - k D, less N if that is >= N/2
+          if (f0 + l - k * D < N / 2) b[1] = max(b[1], m2);
+          else b[0] = max(b[0], m2);
         }
       };
       K::F::run(reinterpret_cast<float4*>(sm), tws, v, free, dst);
@@ -371,7 +372,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
       for (int l = 0; l < 2; ++l)
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-          profile_max(pr + l + h * N, __float_as_uint(A.power == 2 ? best[l][h] : sqrtf(best[l][h])));
+          profile_max(pr + l + h * N, A.power == 2 ? best[l][h] : __float_as_uint(sqrtf(__uint_as_float(best[l][h]))));
     } else {
       // thread t's bin f = i + p j goes to channel kh = i + p ((j + RL / 2) mod RL), position
       // (f0 + N/2 - f D) mod N of its row (even, as are f0, N/2 and D)
