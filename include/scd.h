@@ -336,9 +336,12 @@ SCD_API scd_status scd_stream_advance(scd_batch_plan* plan, void* x_arena, const
  * scd_batch_tune: items of 32..512 KiB, SSCA slots of 8..64 MiB, and the
  *   staged schedules; re-plans `plan` with the fastest setting (plans created later for the
  *   same workload start from it).
- * scd_ssca_tune: the STAGES schedule and the PERSISTENT one with the same knobs, for
- *   (N, Np, opts->precision); later SCD_SCHEDULE_AUTO calls use the fastest.  Arguments as
- *   scd_ssca (opts->workspace at least scd_ssca_workspace_bytes). */
+ * scd_ssca_tune: the STAGES schedule, FUSED where its tiles fit, and the PERSISTENT one with
+ *   the same knobs, for (N, Np, opts->precision); later SCD_SCHEDULE_AUTO calls use the fastest.
+ *   Tuning an FP32 auto estimate of a power-of-two N also times the lag-domain kernels and keeps
+ *   a choice for such estimates beside the one for the cross and conjugate estimates of the sizes;
+ *   tuning a cross or conjugate estimate leaves the auto estimates' choice alone.
+ *   Arguments as scd_ssca (opts->workspace at least scd_ssca_workspace_bytes). */
 SCD_API scd_status scd_batch_tune(scd_batch_plan* plan, const void* x_arena, const float* window, void* out_arena,
                                   void* workspace, void* stream, int32_t reps);
 SCD_API scd_status scd_ssca_tune(const void* x, int64_t N, int32_t Np, const float* window, void* out,

@@ -201,15 +201,15 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
   }
   TuneEntry choice{o.schedule, 0, 0, 0.0};
   const bool automatic = given || o.schedule == SCD_SCHEDULE_AUTO;
-  if (automatic) choice = given ? *given : scd::ssca_auto_choice(N, Np, o.precision);
+  const bool lag = o.precision == SCD_FP32 && !o.y && !conj;
+  if (automatic) choice = given ? *given : scd::ssca_auto_choice(N, Np, o.precision, lag);
   if (choice.schedule != SCD_SCHEDULE_STAGES && choice.schedule != SCD_SCHEDULE_PERSISTENT &&
       choice.schedule != SCD_SCHEDULE_FUSED)
     return SCD_ERR_ARG;
   const bool fused = scd::ssca_fused_supported(N, Np, o.precision);
   // the auto estimate under AUTO or FUSED: the lag-domain kernels (an explicit FUSED where its tiles
   // do not fit asks for the STAGES kernels)
-  if (choice.schedule == SCD_SCHEDULE_FUSED && o.precision == SCD_FP32 && !o.y && !conj &&
-      (fused || automatic)) {
+  if (choice.schedule == SCD_SCHEDULE_FUSED && lag && (fused || automatic)) {
     // events as the fused schedule records them (before, between the strip and the channel transforms,
     // after); at the sizes where AUTO used to run STAGES, one more between the strip's two passes
     StageMarks m{o, fused ? 3 : 4};

@@ -1167,9 +1167,12 @@ scd_batch_plan* single_plan(int64_t N, int Np, int precision, int64_t item, int6
 
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-std::string ssca_key(int64_t N, int Np, int precision) {
+// An FP32 auto estimate of a power-of-two N has kernels of its own under FUSED (ssca_lag.cuh), so it has an
+// entry of its own (lag): one that timed the kernels of the cross and conjugate estimates, or was saved before
+// there were others, says nothing about it.
+std::string ssca_key(int64_t N, int Np, int precision, bool lag) {
   char buf[96];
-  snprintf(buf, sizeof buf, "|ssca|N=%lld|Np=%d|p=%d", (long long)N, Np, precision);
+  snprintf(buf, sizeof buf, "|%s|N=%lld|Np=%d|p=%d", lag ? "ssca-lag" : "ssca", (long long)N, Np, precision);
   return device_key() + buf;
 }
 }  // namespace
@@ -1214,9 +1217,9 @@ scd_status ssca_persistent(const float2* x, const float2* y, bool conj, int64_t 
   return ssca_persistent_tuned(x, y, conj, N, Np, window, out, ws, ws_bytes, st, precision, kItemBytes, kSlotBytes);
 }
 
-TuneEntry ssca_auto_choice(int64_t N, int Np, int precision) {
+TuneEntry ssca_auto_choice(int64_t N, int Np, int precision, bool lag) {
   TuneEntry e;
-  if (tune_lookup(ssca_key(N, Np, precision), &e)) return e;
+  if (tune_lookup(ssca_key(N, Np, precision, lag), &e)) return e;
   return TuneEntry{precision == SCD_FP32 ? SCD_SCHEDULE_FUSED : SCD_SCHEDULE_STAGES, kItemBytes, kSlotBytes, 0.0};
 }
 
@@ -1236,19 +1239,29 @@ extern "C" scd_status scd_ssca_tune(const void* x, int64_t N, int32_t Np, const 
   o.stage_events = nullptr;
   o.n_stage_events = 0;
   cudaStream_t st = (cudaStream_t)o.stream;
+  // of an auto estimate that has lag-domain kernels two choices: its own (best_lag), and the one of the cross
+  // and conjugate estimates of its sizes (best), whose kernels do the same work on any second signal: y = x
+  const bool lag = o.precision == SCD_FP32 && is_pow2(N) && !o.y && !o.conjugate;
   TuneEntry best{SCD_SCHEDULE_STAGES, kItemBytes, kSlotBytes, 3.4e38};
   o.schedule = SCD_SCHEDULE_STAGES;
   float ms = 0.f;
   scd_status s = time_candidate(st, reps, [&]() { return scd_ssca(x, N, Np, window, out, &o); }, &ms);
   if (s != SCD_OK) return s;
   best.ms = ms;
-  if (o.precision == SCD_FP32 && is_pow2(N)) {
-    // what AUTO runs when never tuned: the lag-domain kernels, or the fused ones for a cross or
-    // conjugate estimate
+  TuneEntry best_lag = best;
+  if (ssca_fused_supported(N, Np, o.precision)) {
+    scd_opts f = o;
+    f.schedule = SCD_SCHEDULE_FUSED;
+    if (lag) { f.y = x; f.normalise = 0; }
+    s = time_candidate(st, reps, [&]() { return scd_ssca(x, N, Np, window, out, &f); }, &ms);
+    if (s != SCD_OK) return s;
+    if (ms < best.ms) best = TuneEntry{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, ms};
+  }
+  if (lag) {
     const TuneEntry fused{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, 0.0};
     s = time_candidate(st, reps, [&]() { return ssca_run(x, N, Np, window, out, o, &fused); }, &ms);
     if (s != SCD_OK) return s;
-    if (ms < best.ms) best = TuneEntry{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, ms};
+    if (ms < best_lag.ms) best_lag = TuneEntry{SCD_SCHEDULE_FUSED, kItemBytes, kSlotBytes, ms};
   }
   const int64_t items[] = {64ll << 10, 128ll << 10, 256ll << 10};
   const int64_t slots[] = {8ll << 20, 16ll << 20, 32ll << 20, 64ll << 20};
@@ -1260,7 +1273,9 @@ extern "C" scd_status scd_ssca_tune(const void* x, int64_t N, int32_t Np, const 
       }, &ms);
       if (s != SCD_OK) return s;
       if (ms < best.ms) best = TuneEntry{SCD_SCHEDULE_PERSISTENT, item, slot, ms};
+      if (ms < best_lag.ms) best_lag = TuneEntry{SCD_SCHEDULE_PERSISTENT, item, slot, ms};
     }
-  tune_store(ssca_key(N, Np, o.precision), best);
+  tune_store(ssca_key(N, Np, o.precision, false), best);
+  if (lag) tune_store(ssca_key(N, Np, o.precision, true), best_lag);
   return SCD_OK;
 }

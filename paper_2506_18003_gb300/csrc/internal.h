@@ -131,8 +131,9 @@ struct TuneEntry {
 std::string device_key();                                    // "<GPU name>/sm<cc>"
 bool tune_lookup(const std::string& key, TuneEntry* out);
 void tune_store(const std::string& key, const TuneEntry& e);
-// scd_ssca under SCD_SCHEDULE_AUTO: the tuned choice, else the default (FUSED in the FP32 form)
-TuneEntry ssca_auto_choice(int64_t N, int Np, int precision);
+// scd_ssca under SCD_SCHEDULE_AUTO: the tuned choice, else the default (FUSED in the FP32 form); lag: an
+// estimate that FUSED runs in the lag domain
+TuneEntry ssca_auto_choice(int64_t N, int Np, int precision, bool lag);
 // scd_ssca with the choice AUTO makes given (NULL: from o.schedule, the tuned choice or the default)
 scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, void* out, const scd_opts& o,
                     const TuneEntry* choice);
