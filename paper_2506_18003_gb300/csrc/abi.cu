@@ -174,14 +174,27 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
     window = scd::table_hamming(Np, &e);
     if (!window) return cuda_fail(e);
   }
+  // the choice of schedule, powers of two only
+  const bool pow2 = scd::is_pow2(N), automatic = given || o.schedule == SCD_SCHEDULE_AUTO;
+  const bool lag_form = pow2 && o.precision == SCD_FP32 && !o.y && !conj;
+  TuneEntry choice{o.schedule, 0, 0, 0.0};
+  if (pow2 && automatic) choice = given ? *given : scd::ssca_auto_choice(N, Np, o.precision, lag_form);
+  if (pow2 && choice.schedule != SCD_SCHEDULE_STAGES && choice.schedule != SCD_SCHEDULE_PERSISTENT &&
+      choice.schedule != SCD_SCHEDULE_FUSED)
+    return SCD_ERR_ARG;
+  const bool fused = pow2 && scd::ssca_fused_supported(N, Np, o.precision);
+  // the auto estimate under AUTO or FUSED: the lag-domain kernels (an explicit FUSED where its tiles
+  // do not fit asks for the STAGES kernels)
+  const bool lag = lag_form && choice.schedule == SCD_SCHEDULE_FUSED && (fused || automatic);
+  const float* gain = nullptr;
   if (o.normalise) {
     void* area = (char*)o.workspace + need - scd::norm_workspace_bytes();
-    if ((e = scd::normalised_window((const float2*)x, N, window, Np, o.normalise, 2, area, &window, st)) !=
-        cudaSuccess)
+    if ((e = scd::normalised_window((const float2*)x, N, window, Np, o.normalise, 2, area, &window, st,
+                                    lag ? &gain : nullptr)) != cudaSuccess)
       return cuda_fail(e);
   }
   float2* ws = (float2*)o.workspace;
-  if (!scd::is_pow2(N)) {
+  if (!pow2) {
     // any N, staged kernels only: AUTO takes mixed-radix strips where N has a split (FP32); else, and under an
     // explicit STAGES, which exact-length batch plans equal bit for bit, Bluestein's identity
     const bool smooth = o.schedule == SCD_SCHEDULE_AUTO;
@@ -199,25 +212,15 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
     if ((e = m.mark(3, st)) != cudaSuccess) return cuda_fail(e);
     return SCD_OK;
   }
-  TuneEntry choice{o.schedule, 0, 0, 0.0};
-  const bool automatic = given || o.schedule == SCD_SCHEDULE_AUTO;
-  const bool lag = o.precision == SCD_FP32 && !o.y && !conj;
-  if (automatic) choice = given ? *given : scd::ssca_auto_choice(N, Np, o.precision, lag);
-  if (choice.schedule != SCD_SCHEDULE_STAGES && choice.schedule != SCD_SCHEDULE_PERSISTENT &&
-      choice.schedule != SCD_SCHEDULE_FUSED)
-    return SCD_ERR_ARG;
-  const bool fused = scd::ssca_fused_supported(N, Np, o.precision);
-  // the auto estimate under AUTO or FUSED: the lag-domain kernels (an explicit FUSED where its tiles
-  // do not fit asks for the STAGES kernels)
-  if (choice.schedule == SCD_SCHEDULE_FUSED && lag && (fused || automatic)) {
+  if (lag) {
     // events as the fused schedule records them (before, between the strip and the channel transforms,
     // after); at the sizes where AUTO used to run STAGES, one more between the strip's two passes
     StageMarks m{o, fused ? 3 : 4};
     int mk = 0;
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_strip((const float2*)x, N, Np, ws, (float2*)out, 0, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_strip((const float2*)x, gain, N, Np, ws, (float2*)out, 0, st)) != cudaSuccess) return cuda_fail(e);
     if (!fused && (e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_strip((const float2*)x, N, Np, ws, (float2*)out, 1, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag_strip((const float2*)x, gain, N, Np, ws, (float2*)out, 1, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = scd::ssca_lag_chan(ws, N, Np, window, (float2*)out, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);

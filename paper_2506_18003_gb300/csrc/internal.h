@@ -83,9 +83,11 @@ cudaError_t ssca_fused_rows(const float2* ws, int64_t N, int Np, float2* out, cu
 
 // Auto estimates in the lag domain (ssca_lag.cu, ssca_lag.cuh; FP32 form, N a power of two): strip =
 // lag products and M1-point pass (pass 0, scratch in out), M2-point pass into ws (pass 1); chan = window
-// and Np-point transform over the lags into out[kh][sh].  ws: 8 (Np/2 + 1) N bytes.
+// and Np-point transform over the lags into out[kh][sh].  ws: 8 (Np/2 + 1) N bytes.  gain (device, may be
+// NULL): factor of the lag products (normalised_window).
 bool ssca_lag_tables(int64_t N, int Np, cudaError_t* err);      // builds the tables they use
-cudaError_t ssca_lag_strip(const float2* x, int64_t N, int Np, float2* ws, float2* out, int pass, cudaStream_t st);
+cudaError_t ssca_lag_strip(const float2* x, const float* gain, int64_t N, int Np, float2* ws, float2* out, int pass,
+                           cudaStream_t st);
 cudaError_t ssca_lag_chan(const float2* ws, int64_t N, int Np, const float* window, float2* out, cudaStream_t st);
 
 // Default schedule of scd_ssca: one persistent launch (batch.cu) over a cached one-signal plan.
@@ -144,10 +146,11 @@ scd_status ssca_persistent_tuned(const float2* x, const float2* y, bool conj, in
 // ---------------------------------------------------------------- input normalisation (norm.cu)
 // Window a scaled for the input normalisation of the first n samples of x (mode 1: mean power
 // 1, mode 2: peak magnitude 1; `power` 1 for FAM, 2 for SSCA), written into `area`
-// (norm_workspace_bytes() bytes of device workspace); *window_out points into it.
+// (norm_workspace_bytes() bytes of device workspace); *window_out points into it.  gain not NULL: the
+// window lacks the power of two that *gain then points to.
 size_t norm_workspace_bytes();
 cudaError_t normalised_window(const float2* x, int64_t n, const float* a, int Np, int mode, int power, void* area,
-                              const float** window_out, cudaStream_t st);
+                              const float** window_out, cudaStream_t st, const float** gain = nullptr);
 
 // ---------------------------------------------------------------- diagnostics (diag.cu)
 // Fault injection for tests, from the environment variable SCD_FAULT_INJECT (read on every

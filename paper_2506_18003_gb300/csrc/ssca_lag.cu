@@ -156,11 +156,13 @@ cudaError_t one(const float2* x, int64_t N, int Np, const float* window, float2*
 }
 }  // namespace
 
-cudaError_t ssca_lag_strip(const float2* x, int64_t N, int Np, float2* ws, float2* out, int pass, cudaStream_t st) {
+cudaError_t ssca_lag_strip(const float2* x, const float* gain, int64_t N, int Np, float2* ws, float2* out, int pass,
+                           cudaStream_t st) {
   LagArgs A;
   cudaError_t e = one(x, N, Np, nullptr, ws, out, &A);
   if (e != cudaSuccess) return e;
   if (!(A.tw = table_pass2(pass == 0 ? A.M1 : A.M2, &e))) return e;
+  A.gain = gain;
   count_launches(1);
   return pass == 0 ? lag_cols(A, st) : lag_rows(A, st);
 }

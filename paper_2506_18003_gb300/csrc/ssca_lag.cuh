@@ -80,6 +80,7 @@ struct LagArgs {
   float2* out;
   float* prof;
   const float* window;
+  const float* gain;                                        // factor of the lag products, or nullptr (cols)
   const float2* tw;                                         // pass table of the pass's transform
   const float2* wN;
   unsigned* err;
@@ -171,12 +172,13 @@ __device__ __forceinline__ void lag_cols_tile(unsigned char* sm, const LagArgs& 
 #pragma unroll
   for (int b = 0; b < B; ++b) rot[b] = __ldg(A.wN + m2 * (t + b * T));
   wait_for_previous();
+  const float gain = A.gain ? load_written(A.gain) : 1.f;   // (exact: a power of two)
   C2 v[E];
   const float2* xp = A.x + g.x + (t * M2 + m2);
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int n = r * (M1 / E) * M2;
-    const float2 a = load_written(xp + n);
+    const float2 a = cscale(load_written(xp + n), gain);
     float2 b0, b1;
     if (r < E - 1) {                                        // n + m + 1 < N: the lags are far below N / E
       b0 = load_written(xp + n + m);
