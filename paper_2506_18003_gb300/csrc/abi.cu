@@ -66,6 +66,11 @@ scd_status check_ssca(const void* x, int64_t N, int32_t Np, const float* window,
   return SCD_OK;
 }
 
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t p = (uintptr_t)a, q = (uintptr_t)b;
+  return p < q + nb && q < p + na;
+}
+
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // The variant fields: y (when given) a complex64 device array aligned like x; conjugate 0 / 1.
@@ -184,8 +189,12 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
     return SCD_ERR_ARG;
   const bool fused = pow2 && scd::ssca_fused_supported(N, Np, o.precision);
   // the auto estimate under AUTO or FUSED: the lag-domain kernels (an explicit FUSED where its tiles
-  // do not fit asks for the STAGES kernels)
-  const bool lag = lag_form && choice.schedule == SCD_SCHEDULE_FUSED && (fused || automatic);
+  // do not fit asks for the STAGES kernels).  They use `out` as scratch before they are done with x and the
+  // window; the others write it last, so those serve a caller whose inputs lie in the output's memory.
+  const size_t out_bytes = sizeof(float2) * (size_t)Np * (size_t)N;
+  const bool lag = lag_form && choice.schedule == SCD_SCHEDULE_FUSED && (fused || automatic) &&
+                   !overlap(x, sizeof(float2) * (size_t)N, out, out_bytes) &&
+                   !overlap(window, sizeof(float) * (size_t)Np, out, out_bytes);
   const float* gain = nullptr;
   if (o.normalise) {
     void* area = (char*)o.workspace + need - scd::norm_workspace_bytes();
