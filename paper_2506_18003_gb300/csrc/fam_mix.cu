@@ -1,5 +1,8 @@
 // Plans and launches of the mixed-radix FAM pair transforms and SSCA strips (mix2.cuh).
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "internal.h"
 #include "mix2.cuh"
@@ -125,7 +128,7 @@ static int strip_width(const MixPlan& p) {
   return lc;
 }
 
-// Both factors with a plan (found once per length and thread); the widest tiles, then the fewest passes, then the smallest radix sum.
+// Both factors with a plan; the widest tiles, then the fewest passes, then the smallest radix sum.
 static bool find_strip_plan(int64_t N, StripPlan* best) {
   int64_t score = -1;
   if (N > (int64_t)4096 * 4096 || N > INT32_MAX / 2) return false;
@@ -146,16 +149,32 @@ static bool find_strip_plan(int64_t N, StripPlan* best) {
   return score >= 0;
 }
 
+// The splits of up to 64 lengths, also of those without one: the search takes 20 to 40 us, as long as a small
+// estimate's launches, and a program may take several lengths in turn.  (A call asks three times: the
+// thread's last answer first.)
 bool strip_plan(int64_t N, StripPlan* plan) {
+  constexpr size_t kMost = 64;
+  static std::mutex mu;
+  static std::map<int64_t, std::pair<bool, StripPlan>> kept;
   thread_local int64_t last = 0;
-  thread_local bool found = false;
-  thread_local StripPlan kept;
+  thread_local std::pair<bool, StripPlan> mine;
   if (last != N) {
-    found = find_strip_plan(N, &kept);
+    bool known = false;
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      const auto it = kept.find(N);
+      if ((known = it != kept.end())) mine = it->second;
+    }
+    if (!known) {
+      mine.first = find_strip_plan(N, &mine.second);
+      std::lock_guard<std::mutex> lock(mu);
+      if (kept.size() >= kMost) kept.clear();
+      kept[N] = mine;
+    }
     last = N;
   }
-  if (found) *plan = kept;
-  return found;
+  if (mine.first) *plan = mine.second;
+  return mine.first;
 }
 
 bool prepare_strip(int64_t N, cudaError_t* err) {
