@@ -77,6 +77,15 @@ k_fam_pairs_any(const float2* __restrict__ X, const float2* __restrict__ Y, int 
   fam_pairs_any_cta<MM, TC>(X, Y, Np, P, out, tw, chirp, bh, bmats, err);
 }
 
+// The same kernel held to 128 registers per thread, so that two 256-thread CTAs share an SM.
+template <int MM, bool TC>
+__global__ void __launch_bounds__(TileShape<MM>::NT, 2)
+k_fam_pairs_any_2cta(const float2* __restrict__ X, const float2* __restrict__ Y, int Np, int P,
+                     float2* __restrict__ out, const float2* __restrict__ tw, const float2* __restrict__ chirp,
+                     const float2* __restrict__ bh, const unsigned char* __restrict__ bmats, unsigned* err) {
+  fam_pairs_any_cta<MM, TC>(X, Y, Np, P, out, tw, chirp, bh, bmats, err);
+}
+
 template <class K>
 cudaError_t launch_fam_any_k(K kernel, int smem, int NT, int C, const float2* X, const float2* Y, int Np, int P,
                              float2* out, const float2* tw, const float2* chirp, const float2* bh, TcArgs t,
@@ -88,12 +97,31 @@ cudaError_t launch_fam_any_k(K kernel, int smem, int NT, int C, const float2* X,
   return cudaGetLastError();
 }
 
+// Where the pairs outnumber the SMs, the FP32 form of the cyclic lengths whose CTAs have 256 threads runs two
+// CTAs per SM (microseconds per estimate, one / two: (Np, P) = (64, 4001) 150 / 142, cross 292 / 238; (128, 4001)
+// 566 / 519, cross 1094 / 832); with no more pairs than SMs the uncapped kernel ((16, 4001) 17 / 23).
 template <int MM, bool TC>
 cudaError_t launch_fam_any(const float2* X, const float2* Y, int Np, int P, float2* out, const float2* tw,
                            const float2* chirp, const float2* bh, TcArgs t, cudaStream_t st) {
   using S = TileShape<MM>;
   constexpr int sm = ResidentSmem<MM, TC>::total;
+  if constexpr (!TC && MM >= 4096 && S::NT <= 256) {
+    cudaError_t e;
+    const int sms = sm_count(&e);
+    if (!sms) return e;
+    if (fam_pair_count<0>(Np, X == Y) > (int64_t)sms * S::C)
+      return launch_fam_any_k(k_fam_pairs_any_2cta<MM, TC>, sm, S::NT, S::C, X, Y, Np, P, out, tw, chirp, bh, t, st);
+  }
   return launch_fam_any_k(k_fam_pairs_any<MM, TC>, sm, S::NT, S::C, X, Y, Np, P, out, tw, chirp, bh, t, st);
+}
+
+// At the cyclic length 4096 a pair fills a CTA in the one-pair form and two pairs do in the packed form, which
+// then takes 1.82 times as long.  An SM holds two CTAs of either: the packed form is the better one unless its
+// last round leaves more of the chip idle than it saves (microseconds per estimate, packed / one-pair, auto:
+// (Np, P) = (16, 1999) 14.2 / 10.5, (64, 1777) 58.1 / 54.6; (32, 1999) 20.1 / 24.7, (128, 1999) 196 / 205).
+bool one_pair_is_better(int64_t pairs, int sms) {
+  auto rounds = [&](int64_t ctas) { return ctas <= sms ? (int64_t)1 : 2 * ((ctas + 2 * sms - 1) / (2 * sms)); };
+  return 1.82 * (double)rounds(pairs / 2) > (double)rounds(pairs);
 }
 
 // Two pairs at a time on the packed lanes (bluestein2.cuh): the FP32 form, cyclic lengths 64 .. 4096.
@@ -307,6 +335,12 @@ cudaError_t fam_pair_fft_any(const float2* X, const float2* Y, int Np, int P, fl
     SCD_FA(8, true) SCD_FA(16, true) SCD_FA(32, true) SCD_FA(64, true) SCD_FA(128, true) SCD_FA(256, true)
     SCD_FA(512, true) SCD_FA(1024, true) SCD_FA(2048, true) SCD_FA(4096, true) SCD_FA(8192, true) SCD_FA(16384, true)
     default: return cudaErrorInvalidValue;
+  }
+  if (MM == 4096) {
+    const int sms = sm_count(&err);
+    if (!sms) return err;
+    if (one_pair_is_better(fam_pair_count<0>(Np, X == Y), sms))
+      return launch_fam_any<4096, false>(X, Y, Np, P, out, tw, chirp, bh, t, st);
   }
   switch (MM) {
     SCD_FA(8, false) SCD_FA(16, false) SCD_FA(32, false)
