@@ -246,12 +246,13 @@ SCD_API scd_status scd_batch_plan_create_exact(int32_t estimator, int32_t nsig, 
  *   workspace_bytes      device workspace scd_batch_run needs */
 SCD_API scd_status scd_batch_query(const scd_batch_plan* plan, int64_t* x_offsets, int64_t* out_offsets,
                                    int64_t* sizes, int64_t* used_len, size_t* workspace_bytes);
-/* Enqueues the whole batch on `stream` (a cudaStream_t; with NULL the kernel is launched
- * directly instead of through a graph).  x_arena complex64[x_offsets[nsig]], out_arena
- * complex64[out_offsets[nsig]], window float32[Np] or NULL (Hamming), workspace as queried.
- * Runs of one plan must not overlap in time (they share the plan's counters).  A dependency
- * wait that gives up (bounded at 2 s) sets the device error word: scd_check_device() then
- * returns SCD_ERR_TIMEOUT. */
+/* Enqueues the whole batch on `stream` (a cudaStream_t; with NULL, and for small SSCA plans of one
+ * size whose three launches then take less time, the kernels are launched directly instead of
+ * through a graph).  x_arena complex64[x_offsets[nsig]], out_arena complex64[out_offsets[nsig]],
+ * window float32[Np] or NULL (Hamming), workspace as queried; the buffers must not overlap.
+ * Runs of one plan must not overlap in time (they share the workspace and the plan's counters).
+ * A dependency wait that gives up (bounded at 2 s) sets the device error word:
+ * scd_check_device() then returns SCD_ERR_TIMEOUT. */
 SCD_API scd_status scd_batch_run(scd_batch_plan* plan, const void* x_arena, const float* window, void* out_arena,
                                  void* workspace, void* stream);
 SCD_API void scd_batch_plan_destroy(scd_batch_plan* plan);

@@ -111,6 +111,7 @@ struct scd_batch_plan {
   std::vector<scd::LagSig> lag_sigs;
   std::vector<LagLaunch> lag_launches;
   scd::LagSig* d_lag = nullptr;
+  bool lag_small = false;                 // all of the plan's estimates together would fit L2
   unsigned* d_counters = nullptr;
   int64_t total = 0;
   size_t ws_bytes = 0;
@@ -167,6 +168,18 @@ void free_plan(scd_batch_plan* p) {
   if (p->d_fam) cudaFree(p->d_fam);
   if (p->d_counters) cudaFree(p->d_counters);
   delete p;
+}
+
+// The nodes that the next launch captured on `st` would depend on (none if `st` is not being captured).
+cudaError_t capture_frontier(cudaStream_t st, bool* capturing, std::vector<cudaGraphNode_t>* nodes) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t n = 0;
+  const cudaError_t e = cudaStreamGetCaptureInfo(st, &status, nullptr, nullptr, &deps, &edges, &n);
+  *capturing = e == cudaSuccess && status == cudaStreamCaptureStatusActive;
+  if (*capturing) nodes->assign(deps, deps + n);
+  return e;
 }
 
 scd_status cuda_status(cudaError_t e) {
@@ -357,6 +370,10 @@ scd_status build_tasks(scd_batch_plan* p) {
     };
     // staged == 2: the FP32 SSCA in the lag domain
     const bool lag = !fam && !tc && p->staged == 2;
+    p->lag_small = lag && (int64_t)sizeof(float2) * p->ws_off[nsig] <= (int64_t(128) << 20);
+    // lag pairs of a profile plan's Y, beside R: the persistent schedule's slots (unused here) while they last
+    int64_t y_at = p->ws_off[nsig];
+    const int64_t y_end = (int64_t)(p->ws_bytes / sizeof(float2));
     int f0 = 0;
     for (int i = 0; i < nsig && !lag; ++i) {
       Task t = stage0_task(i);
@@ -405,24 +422,30 @@ scd_status build_tasks(scd_batch_plan* p) {
         LagArgs A{};
         A.N = (int)N; A.M1 = sp.M1; A.M2 = sp.M2; A.Np = Np; A.power = p->prof_power; A.err = p->err;
         const int64_t first = (int64_t)p->lag_sigs.size();
+        const int pairs = lag_pairs(Np);
+        for (int i = 0; i < nsig; ++i) A.nsig += p->sizes[i] == N;
+        // Y where S will be; of profiles in the slots if the class fits there, else behind R, which takes
+        // Np/2 + 1 of the signal's Np rows, half of the lag pairs at a time (Np/2 - 1 rows are left).  (The
+        // second set of strip launches costs a small plan 4 us: one window of 2^13, Np = 64 20.6 -> 14.4 us.)
+        const int64_t y_sig = 2 * pairs * N;
+        const bool slots = p->prof_power && y_at + A.nsig * y_sig <= y_end;
+        const int group = p->prof_power && !slots ? (pairs + 1) / 2 : pairs;
         int64_t r0 = -1;
         for (int i = 0; i < nsig; ++i) {
           if (p->sizes[i] != N) continue;
           if (r0 < 0) r0 = p->ws_off[i];
-          // Y where S will be, or (profiles) behind R, which takes Np/2 + 1 of the signal's Np rows
-          p->lag_sigs.push_back({p->x_off[i], p->prof_power ? p->ws_off[i] + (Np / 2 + 1) * N : p->out_off[i],
-                                 p->ws_off[i], p->out_off[i]});
-          ++A.nsig;
+          int64_t y = p->prof_power ? p->ws_off[i] + (Np / 2 + 1) * N : p->out_off[i];
+          if (slots) { y = y_at; y_at += y_sig; }
+          p->lag_sigs.push_back({p->x_off[i], y, p->ws_off[i], p->out_off[i]});
         }
         if (!(A.wN = table_roots((int)N, &e)) || (e = lag_prepare(sp.M1, sp.M2, Np)) != cudaSuccess) return cuda_status(e);
         auto pass = [&](int kind, int M, int p0, int np) {
           A.p0 = p0; A.np = np;
+          A.clear = p->prof_power && kind == 0 && p0 == 0;
           if (!(A.tw = table_pass2(M, &e))) return cuda_status(e);
           p->lag_launches.push_back({kind, first, r0, A});
           return SCD_OK;
         };
-        // profiles: Y holds half of the lag pairs at a time (Np/2 - 1 rows are left for it)
-        const int pairs = lag_pairs(Np), group = p->prof_power ? (pairs + 1) / 2 : pairs;
         for (int p0 = 0; p0 < pairs; p0 += group) {
           const int np = std::min(group, pairs - p0);
           if ((ls = pass(0, sp.M1, p0, np)) != SCD_OK || (ls = pass(1, sp.M2, p0, np)) != SCD_OK) return ls;
@@ -900,14 +923,24 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   const bool fam = p->estimator == 0, tc = p->precision == SCD_SPLIT_BF16, prof = p->prof_power != 0;
   const int grid = prof ? p->grid_prof : p->grid;
   const size_t cbytes = sizeof(unsigned) * (p->tasks.size() + 1);
-  // profiles are maxima of non-negative values: they start from 0 on every run
-  const size_t pbytes = prof ? sizeof(float) * (size_t)p->out_off[p->nsig] : 0;
+  // profiles are maxima of non-negative values: they start from 0 on every run (the lag-domain column passes
+  // write the zeros themselves)
   // An injected drop is about the persistent launch's waits: a FAM plan on its default schedule runs that
   // launch for it (as its default schedule used to).
   const bool injected = A.drop_task >= 0 && fam && p->staged == 2;
   const bool staged = !injected && (!p->st_launches.empty() || !p->lag_launches.empty());   // (FAM: the channeliser)
+  const size_t pbytes = prof && (!staged || p->lag_launches.empty()) ? sizeof(float) * (size_t)p->out_off[p->nsig] : 0;
+  // Small lag-domain plans are bound by their launches.  Those of one size class go out directly: three
+  // dependent launches, whose set-up then overlaps the run before as well (one signal of 2^14, Np = 64: 16.4
+  // us as a graph, 13.6 so; from 256 MB of estimates on the graph is the faster one by 1 to 4%).  Those of
+  // several classes become graphs with a branch per class, which touch nothing of one another's (four classes
+  // of 2^12 .. 2^15, Np = 64: 52 us in a row, 27 side by side; at 4 GB 2145 and 2328).
+  const bool direct = !st || (staged && p->lag_small && p->lag_launches.size() == 3);
   auto launch_all = [&]() -> cudaError_t {
-    if (!staged) return launch_batch(fam, tc, prof, grid, p->smem, A, st);
+    if (!staged) {                                              // (the staged launches take no work from counters)
+      const cudaError_t em = cudaMemsetAsync(p->d_counters, 0, cbytes, st);
+      return em == cudaSuccess ? launch_batch(fam, tc, prof, grid, p->smem, A, st) : em;
+    }
     for (const auto& L : p->st_launches) {
       cudaError_t el =
           staged_launch(L.kind, L.M, p->Np, tc, L.grid, L.smem, A, p->d_st + L.first, L.count, L.total, st);
@@ -920,7 +953,18 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
       const cudaError_t el = fam2_pairs(G, L.P, true, prof, st);
       if (el != cudaSuccess) return el;
     }
+    bool branches = false;
+    std::vector<cudaGraphNode_t> root;
+    if (p->lag_small && !direct) {
+      const cudaError_t el = capture_frontier(st, &branches, &root);
+      if (el != cudaSuccess) return el;
+    }
     for (const auto& L : p->lag_launches) {
+      if (branches && L.kind == 0 && L.args.p0 == 0) {
+        const cudaError_t el = cudaStreamUpdateCaptureDependencies(st, root.data(), nullptr, root.size(),
+                                                                   cudaStreamSetCaptureDependencies);
+        if (el != cudaSuccess) return el;
+      }
       LagArgs G = L.args;
       G.sig = p->d_lag + L.first;
       G.x = A.x; G.R = A.ws; G.Y = prof ? A.ws : A.out; G.out = A.out; G.prof = (float*)A.out; G.window = w;
@@ -930,9 +974,8 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
     return cudaSuccess;
   };
   count_launches(staged ? (int)(p->st_launches.size() + p->lag_launches.size() + p->fam_launches.size()) : 1);
-  if (!st) {                                                    // legacy stream: no capture, plain launch
-    if ((e = cudaMemsetAsync(p->d_counters, 0, cbytes, st)) != cudaSuccess) return cuda_status(e);
-    if (prof && (e = cudaMemsetAsync(out_arena, 0, pbytes, st)) != cudaSuccess) return cuda_status(e);
+  if (direct) {                                                 // (the legacy stream cannot be captured)
+    if (pbytes && (e = cudaMemsetAsync(out_arena, 0, pbytes, st)) != cudaSuccess) return cuda_status(e);
     e = launch_all();
     return e == cudaSuccess ? SCD_OK : cuda_status(e);
   }
@@ -947,8 +990,7 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
     if (gr->exec) { cudaGraphExecDestroy(gr->exec); *gr = scd_batch_plan::Graph(); }
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return cuda_status(e);
-    cudaError_t e1 = cudaMemsetAsync(p->d_counters, 0, cbytes, st);
-    if (e1 == cudaSuccess && prof) e1 = cudaMemsetAsync(out_arena, 0, pbytes, st);
+    cudaError_t e1 = pbytes ? cudaMemsetAsync(out_arena, 0, pbytes, st) : cudaSuccess;
     cudaError_t e2 = e1 == cudaSuccess ? launch_all() : cudaSuccess;
     e = cudaStreamEndCapture(st, &g);
     if (e1 != cudaSuccess) e = e1;

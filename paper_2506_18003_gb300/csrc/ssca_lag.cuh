@@ -26,8 +26,8 @@
 // the last radix pass and the stores.  Loads through registers instead need L1 lines for every load
 // in flight, which the exchange areas of enough CTAs leave too few of (fft2.cuh's 16 bytes per value
 // and thread: 64 KB per CTA of 256 threads).
-// Y lies in the output's own memory (S is written last) or, for alpha profiles, in two groups of lag
-// pairs behind R in the workspace.  Traffic: the intermediate (4 Np N bytes) out, in, out and in again,
+// Y lies in the output's own memory (S is written last) or, for alpha profiles, in the workspace: beside R, or
+// behind it in two groups of lag pairs.  Traffic: the intermediate (4 Np N bytes) out, in, out and in again,
 // and S out: 3 x 8 Np N bytes, of which only S must reach HBM while the intermediate fits L2.
 #pragma once
 #include "fft2.cuh"
@@ -84,7 +84,7 @@ struct LagArgs {
   const float2* tw;                                         // pass table of the pass's transform
   const float2* wN;
   unsigned* err;
-  int N, M1, M2, nsig, Np, power;
+  int N, M1, M2, nsig, Np, power, clear;                    // clear: the column pass zeroes the profiles
   int p0, np;                                               // lag pairs [p0, p0 + np) (cols, rows)
 };
 __device__ __forceinline__ LagSig lag_sig(const LagArgs& A, int s) {
@@ -195,6 +195,10 @@ __device__ __forceinline__ void lag_cols_tile(unsigned char* sm, const LagArgs& 
     *at_bytes(yo, 16u * (uint32_t)(f * M2 + m2)) = c2_f4(cmul(val, cmul(rot[b], stage[j * C + c])));
   };
   K::F::run(reinterpret_cast<float4*>(sm), tws, v, [] { let_next_start(); }, dst);
+  if (A.clear) {                                            // (here, where the values have left the registers)
+    float* pr = A.prof + lag_sig(A, (int)blockIdx.x / sig_tiles).out;
+    for (int i = tile * K::NT + (int)threadIdx.x; i < 2 * N; i += sig_tiles * K::NT) pr[i] = 0.f;
+  }
 }
 
 // Row pass: persistent over the tiles of C rows (pair, q1).
