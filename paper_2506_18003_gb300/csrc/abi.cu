@@ -224,15 +224,21 @@ scd_status ssca_run(const void* x, int64_t N, int32_t Np, const float* window, v
   if (lag) {
     // events as the fused schedule records them (before, between the strip and the channel transforms,
     // after); at the sizes where AUTO used to run STAGES, one more between the strip's two passes
-    StageMarks m{o, fused ? 3 : 4};
-    int mk = 0;
-    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_strip((const float2*)x, gain, N, Np, ws, (float2*)out, 0, st)) != cudaSuccess) return cuda_fail(e);
-    if (!fused && (e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_strip((const float2*)x, gain, N, Np, ws, (float2*)out, 1, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = scd::ssca_lag_chan(ws, N, Np, window, (float2*)out, st)) != cudaSuccess) return cuda_fail(e);
-    if ((e = m.mark(mk++, st)) != cudaSuccess) return cuda_fail(e);
+    struct Marks {
+      StageMarks m;
+      cudaStream_t st;
+      bool all;
+      int next;
+      cudaError_t mark() { return m.mark(next++, st); }
+    } mk{StageMarks{o, fused ? 3 : 4}, st, !fused, 0};
+    auto between = [](void* ctx, int pass) -> cudaError_t {
+      Marks* k = (Marks*)ctx;
+      return pass == 1 || k->all ? k->mark() : cudaSuccess;
+    };
+    if ((e = mk.mark()) != cudaSuccess) return cuda_fail(e);
+    if ((e = scd::ssca_lag((const float2*)x, gain, N, Np, window, ws, (float2*)out, st, between, &mk)) != cudaSuccess)
+      return cuda_fail(e);
+    if ((e = mk.mark()) != cudaSuccess) return cuda_fail(e);
     return SCD_OK;
   }
   if (choice.schedule == SCD_SCHEDULE_FUSED && fused) {

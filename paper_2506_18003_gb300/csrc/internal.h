@@ -81,14 +81,13 @@ cudaError_t ssca_fused_chancol(const float2* x, const float2* y, bool conj, int6
                                float2* ws, cudaStream_t st);
 cudaError_t ssca_fused_rows(const float2* ws, int64_t N, int Np, float2* out, cudaStream_t st);
 
-// Auto estimates in the lag domain (ssca_lag.cu, ssca_lag.cuh; FP32 form, N a power of two): strip =
-// lag products and M1-point pass (pass 0, scratch in out), M2-point pass into ws (pass 1); chan = window
-// and Np-point transform over the lags into out[kh][sh].  ws: 8 (Np/2 + 1) N bytes.  gain (device, may be
+// Auto estimates in the lag domain (ssca_lag.cu, ssca_lag.cuh; FP32 form, N a power of two): lag products
+// and M1-point pass (scratch in out), M2-point pass into ws, then window and Np-point transform over the lags
+// into out[kh][sh]; between(ctx, p) after passes 0 and 1.  ws: 8 (Np/2 + 1) N bytes.  gain (device, may be
 // NULL): factor of the lag products (normalised_window).
 bool ssca_lag_tables(int64_t N, int Np, cudaError_t* err);      // builds the tables they use
-cudaError_t ssca_lag_strip(const float2* x, const float* gain, int64_t N, int Np, float2* ws, float2* out, int pass,
-                           cudaStream_t st);
-cudaError_t ssca_lag_chan(const float2* ws, int64_t N, int Np, const float* window, float2* out, cudaStream_t st);
+cudaError_t ssca_lag(const float2* x, const float* gain, int64_t N, int Np, const float* window, float2* ws, float2* out,
+                     cudaStream_t st, cudaError_t (*between)(void*, int), void* ctx);
 
 // Default schedule of scd_ssca: one persistent launch (batch.cu) over a cached one-signal plan.
 size_t ssca_persistent_workspace(int64_t N, int Np);

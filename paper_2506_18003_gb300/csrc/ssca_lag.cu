@@ -142,37 +142,25 @@ bool ssca_lag_tables(int64_t N, int Np, cudaError_t* err) {
          device_error_word(err);
 }
 
-namespace {
 // One signal: Y in the output's memory, R in the workspace.
-cudaError_t one(const float2* x, int64_t N, int Np, const float* window, float2* ws, float2* out, LagArgs* A) {
+cudaError_t ssca_lag(const float2* x, const float* gain, int64_t N, int Np, const float* window, float2* ws, float2* out,
+                     cudaStream_t st, cudaError_t (*between)(void*, int), void* ctx) {
   LagSplit s;
   if (!lag_split(N, &s)) return cudaErrorInvalidValue;
-  *A = LagArgs{};
-  A->x = x; A->Y = out; A->R = ws; A->out = out; A->window = window;
-  A->N = (int)N; A->M1 = s.M1; A->M2 = s.M2; A->nsig = 1; A->Np = Np; A->np = lag_pairs(Np);
+  LagArgs A{};
+  A.x = x; A.gain = gain; A.Y = out; A.R = ws; A.out = out; A.window = window;
+  A.N = (int)N; A.M1 = s.M1; A.M2 = s.M2; A.nsig = 1; A.Np = Np; A.np = lag_pairs(Np);
   cudaError_t e;
-  if (!(A->wN = table_roots((int)N, &e)) || !(A->err = device_error_word(&e))) return e;
-  return lag_prepare(s.M1, s.M2, Np);
-}
-}  // namespace
-
-cudaError_t ssca_lag_strip(const float2* x, const float* gain, int64_t N, int Np, float2* ws, float2* out, int pass,
-                           cudaStream_t st) {
-  LagArgs A;
-  cudaError_t e = one(x, N, Np, nullptr, ws, out, &A);
-  if (e != cudaSuccess) return e;
-  if (!(A.tw = table_pass2(pass == 0 ? A.M1 : A.M2, &e))) return e;
-  A.gain = gain;
-  count_launches(1);
-  return pass == 0 ? lag_cols(A, st) : lag_rows(A, st);
-}
-
-cudaError_t ssca_lag_chan(const float2* ws, int64_t N, int Np, const float* window, float2* out, cudaStream_t st) {
-  LagArgs A;
-  cudaError_t e = one(nullptr, N, Np, window, const_cast<float2*>(ws), out, &A);
-  if (e != cudaSuccess) return e;
-  if (!(A.tw = table_pass2(Np, &e))) return e;
-  count_launches(1);
+  const float2 *tw1, *tw2, *twc;
+  if (!(A.wN = table_roots((int)N, &e)) || !(A.err = device_error_word(&e)) || !(tw1 = table_pass2(s.M1, &e)) ||
+      !(tw2 = table_pass2(s.M2, &e)) || !(twc = table_pass2(Np, &e)) || (e = lag_prepare(s.M1, s.M2, Np)) != cudaSuccess)
+    return e;
+  count_launches(3);
+  A.tw = tw1;
+  if ((e = lag_cols(A, st)) != cudaSuccess || (e = between(ctx, 0)) != cudaSuccess) return e;
+  A.tw = tw2;
+  if ((e = lag_rows(A, st)) != cudaSuccess || (e = between(ctx, 1)) != cudaSuccess) return e;
+  A.tw = twc;
   return lag_chan(A, 0, false, st);
 }
 

@@ -74,13 +74,19 @@ void save_locked() {
 }  // namespace
 
 std::string device_key() {
+  static std::mutex mu;
+  static std::map<int, std::string> kept;                       // per device, asked for once
   int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return "unknown";
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = kept.find(dev);
+  if (it != kept.end()) return it->second;
   cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return "unknown";
+  if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return "unknown";
   std::string name = prop.name;
   for (char& c : name)
     if (c == '"' || c == '|') c = '_';
-  return name + "/sm" + std::to_string(prop.major * 10 + prop.minor);
+  return kept[dev] = name + "/sm" + std::to_string(prop.major * 10 + prop.minor);
 }
 
 bool tune_lookup(const std::string& key, TuneEntry* out) {
