@@ -123,16 +123,20 @@ struct LagChan {
   static constexpr int NT = NTHR, C = NTHR / lag_t(NP);
   using F = PairFft<NP, C, kInterleaved>;
   static_assert(C * PI::T == NT, "tile shape");
+  // blocks of CB lane pairs with a per-tile factor each (`turn`): as many lane pairs as a 128-thread tile has, so
+  // that a frequency's factors, and with them the estimate's bits, do not depend on the tile's width
+  static constexpr int BLOCKS = NTHR / 128, CB = C / BLOCKS;
+  static_assert(BLOCKS == 1 || BLOCKS * (NP / 2) == NT, "one thread per block and lag");
   // landing area: R_m of the tile's 2 C frequencies for the lags m < Np/2, and of the 2 C + 2 frequencies
   // from -(c0 + 2 C) for the lags 1 .. Np/2
   static constexpr int pos_row = 2 * C, neg_row = 2 * C + 2;
   static constexpr int neg_off = lag_up128(NP / 2 * pos_row * 8);
   static constexpr int bytes = NP / 2 * (pos_row + neg_row) * 8;
   static constexpr int step_off = lag_up128(lag_max(neg_off + NP / 2 * neg_row * 8, F::smem_f4 * 16));
-  // W_N^{-d S0 i} of a lane pair's offsets d = 2 c, 2 c + 1 at [i][c] (i < r0 / 2); a[Np/2 - l] W_N^{c0 l}
-  // of the tile, l = 1 .. Np/2; a[Np/2 ..]; the pass table
+  // W_N^{-d S0 i} of a lane pair's offsets d = 2 (c mod CB) and d + 1 at [i][c] (i < r0 / 2); a[Np/2 - l] W_N^{f l}
+  // of each block's first frequency f, l = 1 .. Np/2; a[Np/2 ..]; the pass table
   static constexpr int turn_off = step_off + PI::r0 / 2 * C * 16;
-  static constexpr int win_off = turn_off + NP / 2 * 8;
+  static constexpr int win_off = turn_off + BLOCKS * NP / 2 * 8;
   static constexpr int tw_off = win_off + NP / 2 * 4;
   static constexpr int mbar_off = tw_off + PI::tw_len() * 8;
   static constexpr int smem = mbar_off + 16;
@@ -277,11 +281,12 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
   float* win = reinterpret_cast<float*>(sm + K::win_off);
   float2* tws = reinterpret_cast<float2*>(sm + K::tw_off);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + K::mbar_off);
-  // The factor of lag -l at frequency c0 + d is a[Np/2 - l] W_N^{c0 l} W_N^{d l}: the first two are one
-  // value per lag and tile (thread l - 1 fetches the next tile's root under this tile's last pass), the
-  // last is the same for every tile, u W_N^{-d S0 i} for the thread's l = mh - i S0.  (One root gathered
+  // The factor of lag -l at frequency f + d, f the first of its block, is a[Np/2 - l] W_N^{f l} W_N^{d l}: the
+  // first two are one value per lag and block (a thread of its own fetches the next tile's root under this
+  // tile's last pass), the last is the same for every block, u W_N^{-d S0 i} for the thread's l = mh - i S0.  (One root gathered
   // per lag and frequency instead costs 24 scattered reads per lane pair: N = 2^20, Np = 256 1012 us.)
-  const int lag = (int)threadIdx.x + 1;
+  constexpr int CB = K::CB;
+  const int blk = K::BLOCKS > 1 ? (int)threadIdx.x / H : 0, lag = (int)threadIdx.x - blk * H + 1;
   const float alag = lag <= H ? __ldg(A.window + H - lag) : 0.f;
   // tiles from both ends in turn: tile b's mirrored frequencies are tile sig_tiles - 1 - b's, read while
   // they are still in L2
@@ -289,9 +294,10 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
     const int b = tile % sig_tiles;
     return (b & 1 ? sig_tiles - 1 - (b >> 1) : b >> 1) * (2 * C);
   };
-  auto root = [&](int tile) { return __ldg(A.wN + ((c0_of(tile) * lag) & (N - 1))); };
+  auto root = [&](int tile) { return __ldg(A.wN + (((c0_of(tile) + 2 * CB * blk) * lag) & (N - 1))); };
   const int mh = H - t;
-  const C2 u = c2_pack(__ldg(A.wN + 2 * c * mh), __ldg(A.wN + (2 * c + 1) * mh));
+  const int cb = K::BLOCKS > 1 ? c % CB : c;
+  const C2 u = c2_pack(__ldg(A.wN + 2 * cb * mh), __ldg(A.wN + (2 * cb + 1) * mh));
   auto issue = [&](int tile) {                              // thread 0
     const int s = tile / sig_tiles, c0 = c0_of(tile);
     mbar_expect_tx(mbar, K::bytes);
@@ -305,7 +311,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
   for (int e = threadIdx.x; e < PI::tw_len(); e += K::NT) tws[e] = __ldg(A.tw + e);
   for (int e = threadIdx.x; e < H; e += K::NT) win[e] = __ldg(A.window + H + e);
   for (int e = threadIdx.x; e < E / 2 * C; e += K::NT) {
-    const int d = 2 * (e % C), l = S0 * (e / C);
+    const int d = 2 * (e % CB), l = S0 * (e / C);            // (C is a multiple of CB)
     const float2 s0 = __ldg(A.wN + ((-d * l) & (N - 1))), s1 = __ldg(A.wN + ((-(d + 1) * l) & (N - 1)));
     step[e] = make_float4(s0.x, s1.x, s0.y, s1.y);
   }
@@ -318,7 +324,7 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int c0 = c0_of(tile), f0 = c0 + 2 * c;
     const LagSig g = lag_sig(A, tile / sig_tiles);
-    if (lag <= H) turn[lag - 1] = cscale(next, alag);
+    if (lag <= H) turn[blk * H + lag - 1] = cscale(next, alag);
     const bool got = umma::mbar_wait_bounded(mbar, phase, kMbarPollLimit);
     if (__syncthreads_or(!got)) { ok = false; break; }      // one decision for the whole CTA
     if (tile + (int)gridDim.x >= tiles) let_next_start();   // this CTA's last tile
@@ -337,12 +343,13 @@ __device__ __forceinline__ void lag_chan_cta(unsigned char* sm, const LagArgs& A
       const float2* neg = reinterpret_cast<const float2*>(sm + K::neg_off) + (mh - 1) * K::neg_row + 2 * (C - c);
       const bool wrap = f0 == 0;                            // -0 is frequency 0, not N
       const float2* r0p = A.R + g.r + (int64_t)mh * N;
+      const float2* mine = turn + (K::BLOCKS > 1 ? c / CB * H : 0) + mh - 1;
 #pragma unroll
       for (int i = 0; i < E / 2; ++i) {
         float2 r0 = neg[-i * S0 * K::neg_row];
         const float2 r1 = neg[-i * S0 * K::neg_row - 1];
         if (wrap) r0 = load_written(r0p - i * S0 * N);
-        const C2 f = cmul(i ? cmul(u, take2(step + i * C + c)) : u, turn[mh - 1 - i * S0]);
+        const C2 f = cmul(i ? cmul(u, take2(step + i * C + c)) : u, mine[-i * S0]);
         v[E / 2 + i] = c2_pack(cmulc(c2_lane0(f), r0), cmulc(c2_lane1(f), r1));
       }
     }
