@@ -24,10 +24,12 @@ k_lag_chan(const LagArgs A, const __grid_constant__ CUtensorMap tp, const __grid
   lag_chan_cta<NP, NTHR, PROF>(lag_sm, A, &tp, &tn);
 }
 
-// persistent CTAs of a launch over `tiles` tiles: per_sm of nt threads on every SM, of a large output at
+bool large(const LagArgs& A) { return lag_large(A.N, A.Np, A.nsig, A.power != 0); }
+
+// persistent CTAs of a launch over `tiles` tiles: per_sm of nt threads on every SM, of a large launch at
 // most 512 threads
 cudaError_t grid_of(const LagArgs& A, int64_t tiles, int per_sm, int nt, unsigned* grid) {
-  if (lag_large(A.N, A.Np, A.nsig) && per_sm * nt > 512) per_sm = 512 / nt;
+  if (large(A) && per_sm * nt > 512) per_sm = 512 / nt;
   cudaError_t e;
   const int sms = sm_count(&e);
   if (!sms) return e;
@@ -41,7 +43,7 @@ template <int M1>
 cudaError_t launch_cols(const LagArgs& A, cudaStream_t st) {
   const int64_t tiles = (int64_t)lag_cols_tiles(A.np, M1, A.M2) * A.nsig;
   if (tiles >= (int64_t)0x7FFFFFFF) return cudaErrorInvalidValue;
-  return launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_cols<M1>, (unsigned)tiles, LagCols<M1>::NT, LagCols<M1>::smem, st, A);
+  return launch_dependent(!large(A), k_lag_cols<M1>, (unsigned)tiles, LagCols<M1>::NT, LagCols<M1>::smem, st, A);
 }
 
 template <int M2>
@@ -52,7 +54,7 @@ cudaError_t launch_rows(const LagArgs& A, cudaStream_t st) {
   unsigned grid;
   cudaError_t e = grid_of(A, tiles, K::minb, K::NT, &grid);
   if (e != cudaSuccess) return e;
-  return launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_rows<M2>, grid, K::NT, K::smem, st, A);
+  return launch_dependent(!large(A), k_lag_rows<M2>, grid, K::NT, K::smem, st, A);
 }
 
 template <int NP, int NTHR>
@@ -69,8 +71,8 @@ cudaError_t launch_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st
   const cuuint32_t bp[3] = {K::pos_row, NP / 2, 1}, bn[3] = {K::neg_row, NP / 2, 1};
   if ((e = encode_map_c64(&tp, A.R + r0, 3, dims, strides, bp)) != cudaSuccess) return e;
   if ((e = encode_map_c64(&tn, A.R + r0, 3, dims, strides, bn)) != cudaSuccess) return e;
-  return prof ? launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_chan<NP, NTHR, true>, grid, K::NT, K::smem, st, A, tp, tn)
-              : launch_dependent(!lag_large(A.N, A.Np, A.nsig), k_lag_chan<NP, NTHR, false>, grid, K::NT, K::smem, st, A, tp, tn);
+  return prof ? launch_dependent(!large(A), k_lag_chan<NP, NTHR, true>, grid, K::NT, K::smem, st, A, tp, tn)
+              : launch_dependent(!large(A), k_lag_chan<NP, NTHR, false>, grid, K::NT, K::smem, st, A, tp, tn);
 }
 
 }  // namespace
@@ -130,7 +132,7 @@ cudaError_t lag_chan(const LagArgs& A, int64_t r0, bool prof, cudaStream_t st) {
     case 64: return launch_chan<64, 128>(A, r0, prof, st);
     case 128: return launch_chan<128, 128>(A, r0, prof, st);
     case 256:
-      return lag_large(A.N, 256, A.nsig) ? launch_chan<256, 256>(A, r0, prof, st) : launch_chan<256, 128>(A, r0, prof, st);
+      return large(A) ? launch_chan<256, 256>(A, r0, prof, st) : launch_chan<256, 128>(A, r0, prof, st);
     default: return cudaErrorInvalidValue;
   }
 }

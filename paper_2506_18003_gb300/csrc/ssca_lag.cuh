@@ -62,10 +62,18 @@ __host__ __device__ constexpr int lag_resident(int smem, int by_regs) {
   const int by_smem = 227 * 1024 / (smem + 1024);
   return by_smem < by_regs ? by_smem : by_regs;
 }
-// A launch whose output outgrows L2 (129 MB) keeps at most 512 threads per SM: fewer tiles in flight leave
-// the lines that several of them share in L2 (512-signal batch 14.5 -> 12.8 ms), where a smaller one gains
-// 5% from the full number (N = 2^16, Np = 256 86 -> 82 us).
-inline bool lag_large(int64_t N, int Np, int nsig) { return 8 * N * Np * nsig > (int64_t(256) << 20); }
+// Large launches go out the ordinary way with at most 512 threads per SM, at Np = 256 in tiles of 256 threads:
+// fewer tiles in flight leave the lines that several of them share in L2, and longer runs of S go to memory.
+// Smaller ones gain more from early launch and full SMs.  Microseconds in the two forms, capped / full:
+// estimates, line at 256 MB of S: 2^15 x 64, 8 signals (128 MB) 93 / 76, 17 (272 MB) 178 / 164; between 256 MB and
+// 1 GB the short N favour the full form and the long ones the capped one, by up to 7% either way (2^15 x 64, 24
+// signals 244 / 229; 2^18 x 256 360 / 369; 2^19 x 128 352 / 362); above, 2^18 x 128, 8 (2 GB) 1322 / 1460, 2^20 x 256
+// (2 GB) 1443 / 1717.  Alpha profiles, which write the intermediate alone, half of S, line at 1 GB of it:
+// 2^15 x 64, 17 windows (136 MB) 168 / 151; 2^16 x 256, 8 (512 MB) 576 / 549; 2^18 x 128, 8 (1 GB) 1237 / 1229; 512
+// signals of 2^12 .. 2^18, Np = 128 (classes of up to 5 GB) 11.5 / 12.0 ms.
+inline bool lag_large(int64_t N, int Np, int nsig, bool prof) {
+  return prof ? 4 * N * Np * nsig > (int64_t(1) << 30) : 8 * N * Np * nsig > (int64_t(256) << 20);
+}
 
 // What the three passes of one launch share: nsig signals of one size N, signal s at the given offsets
 // of the arenas (one signal: sig = nullptr, every offset 0).
