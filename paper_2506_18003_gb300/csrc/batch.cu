@@ -937,10 +937,11 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   // of 2^12 .. 2^15, Np = 64: 52 us in a row, 27 side by side; at 4 GB 2145 and 2328).
   const bool direct = !st || (staged && p->lag_small && p->lag_launches.size() == 3);
   auto launch_all = [&]() -> cudaError_t {
-    if (!staged) {                                              // (the staged launches take no work from counters)
-      const cudaError_t em = cudaMemsetAsync(p->d_counters, 0, cbytes, st);
-      return em == cudaSuccess ? launch_batch(fam, tc, prof, grid, p->smem, A, st) : em;
-    }
+    cudaError_t em = cudaSuccess;
+    if (!staged) em = cudaMemsetAsync(p->d_counters, 0, cbytes, st);   // (the staged launches take no work from them)
+    if (em == cudaSuccess && pbytes) em = cudaMemsetAsync(out_arena, 0, pbytes, st);
+    if (em != cudaSuccess) return em;
+    if (!staged) return launch_batch(fam, tc, prof, grid, p->smem, A, st);
     for (const auto& L : p->st_launches) {
       cudaError_t el =
           staged_launch(L.kind, L.M, p->Np, tc, L.grid, L.smem, A, p->d_st + L.first, L.count, L.total, st);
@@ -975,7 +976,6 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   };
   count_launches(staged ? (int)(p->st_launches.size() + p->lag_launches.size() + p->fam_launches.size()) : 1);
   if (direct) {                                                 // (the legacy stream cannot be captured)
-    if (pbytes && (e = cudaMemsetAsync(out_arena, 0, pbytes, st)) != cudaSuccess) return cuda_status(e);
     e = launch_all();
     return e == cudaSuccess ? SCD_OK : cuda_status(e);
   }
@@ -990,11 +990,9 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
     if (gr->exec) { cudaGraphExecDestroy(gr->exec); *gr = scd_batch_plan::Graph(); }
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return cuda_status(e);
-    cudaError_t e1 = pbytes ? cudaMemsetAsync(out_arena, 0, pbytes, st) : cudaSuccess;
-    cudaError_t e2 = e1 == cudaSuccess ? launch_all() : cudaSuccess;
+    const cudaError_t e1 = launch_all();
     e = cudaStreamEndCapture(st, &g);
     if (e1 != cudaSuccess) e = e1;
-    if (e2 != cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&gr->exec, g, 0);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) { gr->exec = nullptr; return cuda_status(e); }
