@@ -1259,7 +1259,7 @@ scd_status ssca_persistent(const float2* x, const float2* y, bool conj, int64_t 
 
 TuneEntry ssca_auto_choice(int64_t N, int Np, int precision, bool lag) {
   TuneEntry e;
-  if (tune_lookup(ssca_key(N, Np, precision, lag), &e)) return e;
+  if (tune_any() && tune_lookup(ssca_key(N, Np, precision, lag), &e)) return e;
   return TuneEntry{precision == SCD_FP32 ? SCD_SCHEDULE_FUSED : SCD_SCHEDULE_STAGES, kItemBytes, kSlotBytes, 0.0};
 }
 

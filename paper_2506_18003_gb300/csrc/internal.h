@@ -130,6 +130,7 @@ struct TuneEntry {
   double ms;              // measured time of the choice
 };
 std::string device_key();                                    // "<GPU name>/sm<cc>"
+bool tune_any();                                             // is there any entry (a call without builds no key)
 bool tune_lookup(const std::string& key, TuneEntry* out);
 void tune_store(const std::string& key, const TuneEntry& e);
 // scd_ssca under SCD_SCHEDULE_AUTO: the tuned choice, else the default (FUSED in the FP32 form); lag: an

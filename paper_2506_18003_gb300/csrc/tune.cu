@@ -89,6 +89,12 @@ std::string device_key() {
   return kept[dev] = name + "/sm" + std::to_string(prop.major * 10 + prop.minor);
 }
 
+bool tune_any() {
+  std::lock_guard<std::mutex> lock(g_mu);
+  load_locked();
+  return !g_cache.empty();
+}
+
 bool tune_lookup(const std::string& key, TuneEntry* out) {
   std::lock_guard<std::mutex> lock(g_mu);
   load_locked();
