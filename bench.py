@@ -229,7 +229,7 @@ def _oracle_worker_init_probe(_):
 
 
 class BatchWorkload:
-    """512 mixed signals through the batched FAM and SSCA (one persistent launch each)."""
+    """512 mixed signals through the batched FAM and SSCA (one plan each)."""
     name = "batch"
     FAM_NP, FAM_L, SSCA_NP = 64, 16, 128
     stages = ["fam_batch", "ssca_batch"]
@@ -948,7 +948,7 @@ def measure_variants(torch, binding, dev, stream, reps=10, warmup=2):
         out[name] = {"ms_per_group": round(ms, 5), "windows_per_group": nwin, "window": W, "hop": hop, "Np": Npw,
                      "stream_msamples_per_s": round(nwin * hop / (ms * 1e-3) / 1e6, 2),
                      "hbm_frac": round(nbytes / (ms * 1e-3) / 1e9 / hbm, 4),
-                     "timed": "host-to-device copy of the group's new samples + the persistent launch"}
+                     "timed": "host-to-device copy of the group's new samples + the plan's run"}
         plan.close()
         del arena, sout, sws
         torch.cuda.empty_cache()

@@ -71,8 +71,10 @@ typedef enum { SCD_FP32 = 0, SCD_SPLIT_BF16 = 1 } scd_precision;
  *   (in this process, or from the SCD_TUNE_CACHE file); if never tuned, in the FP32 form the
  *   lag-domain kernels for an auto estimate of any power-of-two N, else FUSED where it fits,
  *   else STAGES.  An N that is not a power of two runs STAGES by Bluestein's identity, and under
- *   AUTO in the FP32 form, where N is a product of two factors of radices 2 .. 16, mixed-radix
- *   strip transforms. */
+ *   AUTO in the FP32 form mixed-radix strip transforms, where N is a product of two factors of
+ *   17 .. 4096, each a product of at most four radices out of 2 .. 10, 12, 15 and 16 (an N with a
+ *   prime factor above 7 has none).  An auto estimate whose x or window lies in the memory of
+ *   `out` runs the kernels of a cross estimate. */
 typedef enum {
   SCD_SCHEDULE_AUTO = 0,
   SCD_SCHEDULE_STAGES = 1,
@@ -226,10 +228,10 @@ SCD_API scd_status scd_batch_plan_create(int32_t estimator, int32_t nsig, const 
                                          int32_t L, int32_t precision, scd_batch_plan** out);
 /* Exact-length plan: no sample is dropped.  Per-signal sizes FAM P_i = floor((len_i - Np)/L) + 1
  * (>= 2; at most 8192 unless a power of two <= 16384) and SSCA N_i = len_i (>= 4096; at most 2^19
- * unless a power of two <= 2^20); sizes that are not powers of two run by Bluestein's identity
- * (as scd_fam / scd_ssca).  scd_batch_run then runs each signal's estimate with the
- * single-estimate kernels, one signal after the other on the stream (plain launches, no graph;
- * the workspace is the largest single estimate's, from scd_batch_query).  Full estimates only:
+ * unless a power of two <= 2^20); sizes that are not powers of two run by Bluestein's identity.
+ * scd_batch_run then runs one launch per stage and transform size over all signals, in a CUDA
+ * graph; SSCA estimates equal scd_ssca's under SCD_SCHEDULE_STAGES bit for bit, the others agree
+ * with the single calls within the form's rounding.  Full estimates only:
  * scd_batch_plan_set_output(plan, 1 or 2) and scd_batch_plan_set_schedule(plan, STAGES or
  * PERSISTENT) give SCD_ERR_UNSUPPORTED; scd_batch_tune runs once.  The tables of every size
  * are built here, so runs allocate nothing.  Errors as scd_batch_plan_create, and

@@ -40,8 +40,9 @@ const scd_opts& opts_or_default(const scd_opts* o) { return o ? *o : kDefaultOpt
 
 bool np_ok(int32_t Np) { return Np >= 16 && Np <= 256 && scd::is_pow2(Np); }
 
-// Sizes that are not powers of two run on Bluestein's identity with transforms of size
-// M >= 2n - 1: FAM pairs in one CTA (M <= 16384), SSCA four-step transforms (M <= 2^20).
+// Limits of the sizes that are not powers of two, those of Bluestein's identity with transforms of size
+// M >= 2n - 1: FAM pairs in one CTA (M <= 16384), SSCA four-step transforms (M <= 2^20).  (Mixed radices carry
+// many of them in the FP32 form, mix2.cuh.)
 constexpr int32_t kMaxAnyP = 8192;
 constexpr int64_t kMaxAnyN = int64_t(1) << 19;
 

@@ -781,8 +781,8 @@ scd_status build_exact(scd_batch_plan* p) {
 }
 
 // Exact-length plan: every signal's estimate at the sizes its length gives (FAM P_i =
-// floor((len_i - Np)/L) + 1, SSCA N_i = len_i), run with the single-estimate kernels (Bluestein's
-// identity for the sizes that are not powers of two) one signal after the other on the stream.
+// floor((len_i - Np)/L) + 1, SSCA N_i = len_i), one launch per stage and transform size (Bluestein's
+// identity for the sizes that are not powers of two), in one graph.
 scd_status plan_create_exact(int32_t estimator, int32_t nsig, const int64_t* lengths, int32_t Np, int32_t L,
                              int32_t precision, scd_batch_plan** out) {
   using namespace scd;
@@ -925,8 +925,8 @@ scd_status scd_batch_run(scd_batch_plan* p, const void* x_arena, const float* wi
   const size_t cbytes = sizeof(unsigned) * (p->tasks.size() + 1);
   // profiles are maxima of non-negative values: they start from 0 on every run (the lag-domain column passes
   // write the zeros themselves)
-  // An injected drop is about the persistent launch's waits: a FAM plan on its default schedule runs that
-  // launch for it (as its default schedule used to).
+  // An injected drop (a test of the persistent launch's waits) makes a FAM plan on its default schedule, which has
+  // no waits, run that launch, its default of before; SSCA plans are asked for it by set_schedule.
   const bool injected = A.drop_task >= 0 && fam && p->staged == 2;
   const bool staged = !injected && (!p->st_launches.empty() || !p->lag_launches.empty());   // (FAM: the channeliser)
   const size_t pbytes = prof && (!staged || p->lag_launches.empty()) ? sizeof(float) * (size_t)p->out_off[p->nsig] : 0;

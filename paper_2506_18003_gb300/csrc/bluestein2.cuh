@@ -11,7 +11,8 @@
 // (M = 2048) 178 M warp instructions at 0.46 of the issue slots, 16 warps per SM (128 registers; the
 // one-pair form issued 296 M).  Microseconds per estimate, one-pair form / this one:
 //   (Np, P) = (64, 20) 10.7 / 5.7, (64, 100) 10.7 / 7.6, (128, 200, cross) 60 / 35, (64, 333) 21.7 / 15.0,
-//   (256, 500) 213 / 146, (256, 1000) 357 / 313, (64, 1025) 52.7 / 51.7, (128, 1999) 205 / 192.
+//   (256, 500) 213 / 146, (256, 1000) 357 / 313, (32, 1999) 24.7 / 20.2, (128, 1999) 205 / 196.
+// At M = 4096 the one-pair form stays where few pairs leave the packed form's last round short (bluestein.cu).
 // M < 64 (P <= 16) and M > 4096 stay with the one-pair form: the first has too few values for a two-pass
 // plan with equal ends, the second exceeds the 16 x 16 x 16 plan.
 #pragma once
@@ -21,9 +22,6 @@
 
 namespace scd {
 
-#ifndef A2_NT
-#define A2_NT 256
-#endif
 template <int M>
 struct FamAny2 {
   using PI = Plan2Info<M, PlanSym>;

@@ -12,7 +12,7 @@
 // Bound: a transform reads two rows of X (L2) and writes two rows of S (8 P bytes each); GB300's L2 takes
 // 6.3 TB/s of writes alone and 5.1-5.7 TB/s of each with as many reads.  So the kernel is persistent with
 // its twiddle factors in shared memory, and issues 40% fewer instructions than the scalar transform.
-// P = 1024, Np = 256: 111 us for 537 MB of estimates (4.9 TB/s), from 142; what bounds it now is the
+// P = 1024, Np = 256: 104 us for 537 MB of estimates (5.2 TB/s), from 142; what bounds it now is the
 // shared-memory pipe (77% of its cycles) with 16 warps per SM.
 #pragma once
 #include "fft2.cuh"

@@ -88,7 +88,7 @@ bool prepare_mix(int P, cudaError_t* err) {
 // Units per tile: as many as keep the block's threads busy in every pass, but not so many that the last
 // wave of tiles is short of work.  The estimate of a tile's time is the rounds of butterflies per thread,
 // weighted by the radix, and a constant for barriers and set-up.  The limit is half an SM's shared memory (two
-// blocks): at 84 and 60 KB, with more L1 left, Np = 256, P = 1000 takes 151 and 166 us instead of 146.
+// blocks): at 84 and 60 KB, with more L1 left, Np = 256, P = 1000 took 151 and 166 us instead of 146.
 static int mix_units(const MixPlan& p, int64_t units, int slots) {
   int best = 1;
   double cost = 1e30;

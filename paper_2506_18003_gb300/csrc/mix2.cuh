@@ -1,6 +1,7 @@
 // Mixed-radix transforms on the packed lanes: the SSCA strips of a length that splits into two factors with
 // such a plan (17 .. 4096 each), and the FAM pair transform for a P of at most 4096 that is not a
-// power of two but a product of up to four radices 2 .. 16 (every P = 2^a 3^b 5^c 7^d with few exceptions),
+// power of two but a product of up to four radices out of 2 .. 10, 12, 15 and 16 (P = 2^a 3^b 5^c 7^d; lengths
+// with a larger prime factor, 11 x 11 or 11 x 13 for instance, have no plan),
 // FP32 form.  One transform of size P per pair, where Bluestein's identity (bluestein2.cuh) takes two of
 // size >= 2 P - 1.
 //
@@ -14,13 +15,13 @@
 // without twiddle factors by the prime-factor mapping (I. J. Good, 1958), 9 as 3 x 3.
 // Blocks of first digit k_0 lie at an odd stride: the last pass, whose threads run over k_0 first so that
 // its stores are contiguous, then reads 16-byte values from 8 different banks per quarter-warp.
-// Bound by the writes into L2 and the latency of the row reads: at Np = 256, P = 1000 (radices 10, 10, 10)
-// 58.7 M warp instructions at 0.35 of the issue slots, 851 MB written into L2 at 5.8 TB/s (of 6.3 that L2
-// takes; 524 MB are results, the rest partial sectors of the mirrored rows and register spills).
+// Bound by latency: at Np = 256, P = 1000 (radices 10, 10, 10) the 524 MB of results leave at 3.7 TB/s (L2 takes
+// 6.3) with 0.35 of the issue slots used; 16 warps per SM wait on the row reads (a first-pass butterfly
+// of radix 10 issues 40 of 8 bytes) and at the barriers between the passes.
 // Microseconds per estimate, Bluestein one-pair / packed Bluestein / this:
 //   (Np, P) = (64, 20) 10.8 / 5.7 / 6.1, (32, 45) 12.7 / 6.5 / 6.0, (64, 100) 10.6 / 7.6 / 6.2,
-//   (128, 200, cross) 60 / 35 / 22, (256, 500) 213 / 146 / 86, (256, 1000) 357 / 313 / 146,
-//   (128, 1000, cross) 180 / 153 / 65, (64, 1500) 56 / - / 21, (64, 3000) 132 / - / 45, (64, 4050) 144 / - / 57.
+//   (128, 200, cross) 60 / 35 / 21, (256, 500) 213 / 146 / 82, (256, 1000) 357 / 313 / 142,
+//   (128, 1000, cross) 180 / 153 / 66, (64, 1500) 56 / - / 20, (64, 3000) 132 / - / 45, (64, 4050) 144 / - / 56.
 #pragma once
 #include "fft2.cuh"
 #include "pdl.cuh"

@@ -239,7 +239,8 @@ __device__ __forceinline__ void lag_rows_cta(unsigned char* sm, const LagArgs& A
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const bool got = umma::mbar_wait_bounded(mbar, phase, kMbarPollLimit);
     if (__syncthreads_or(!got)) { ok = false; break; }      // one decision for the whole CTA
-    if (tile + (int)gridDim.x >= tiles) let_next_start();   // this CTA's last tile
+    // this CTA's last tile (not before the wait: the channel pass reads the window before its own)
+    if (tile + (int)gridDim.x >= tiles) let_next_start();
     phase ^= 1u;
     C2 v[E];
     {

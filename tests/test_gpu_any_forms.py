@@ -39,3 +39,27 @@ def test_forms_match_oracle(torch, Np, P, variant):
     ref = orc.fam_pairs(x, a, Np, L, P, kh, lh, **okw)
     got = S[torch.from_numpy(kh).cuda(), torch.from_numpy(lh).cuda()].cpu().numpy()
     assert float(np.max(np.abs(got - ref))) / S.abs().max().item() <= FP32_TOL
+
+
+@pytest.mark.parametrize("P", [121, 143])
+def test_fam_factors_without_a_radix(torch, P):
+    """11 and 13 are no radices: products of them run by Bluestein's identity."""
+    Np, L = 32, 8
+    x = signals.modulated("qpsk", (P - 1) * L + Np, 4, 0.1, 5.0, seed=9500 + P)
+    a = orc.hamming_window(Np)
+    S = binding.scd_fam(torch.from_numpy(x).cuda(), Np, L, P)
+    binding.scd_check_device()
+    ref = orc.fam(x, a, Np, L, P)
+    assert float(np.max(np.abs(S.cpu().numpy() - ref)) / np.max(np.abs(ref))) <= FP32_TOL
+
+
+def test_ssca_factors_without_a_radix(torch):
+    """12100 = 110 x 110: the default equals the explicit staged schedule, Bluestein's strips."""
+    N, Np = 12100, 32
+    x = torch.from_numpy(signals.modulated("qpsk", N, 4, 0.1, 5.0, seed=9600)).cuda()
+    S = binding.scd_ssca(x, Np)
+    assert torch.equal(S, binding.scd_ssca(x, Np, schedule="stages"))
+    ch = np.array([0, 15, 16, 31])
+    ref = orc.ssca(x.cpu().numpy(), orc.hamming_window(Np), Np, channels=ch)
+    got = S[torch.from_numpy(ch).cuda()].cpu().numpy()
+    assert float(np.max(np.abs(got - ref))) / S.abs().max().item() <= FP32_TOL
